@@ -63,7 +63,8 @@ typedef enum {
 
 typedef enum {
   /* fused multiply-adds, one division per reconstruction, restricted stencils take the
-   * linear weights directly: agrees with the literal arithmetic to rounding */
+   * linear weights directly, an Euler interface whose stencils are all proven central takes the
+   * central flux of f: agrees with the literal arithmetic to rounding */
   WT_MODE_FAST = 0,
   /* every operation in the order the paper prints it, no contraction: reproduces a
    * literal binary64 evaluation bit for bit */
@@ -75,8 +76,8 @@ typedef enum {
  * it lets a caller compare the launch strategies on its own problems. */
 typedef enum {
   /* chosen from how the grid's tiles fit the device: the step-blocked persistent kernel when
-   * at most one 27-cell (Euler) or 51-cell (scalar) tile per SM is needed, else the
-   * persistent kernel when every tile is co-resident, else the next */
+   * at most one 27-cell (Euler; 9 or 18 cells where those fit too) or 51-cell (scalar) tile
+   * per SM is needed, else the persistent kernel when every tile is co-resident, else the next */
   WT_LAUNCH_AUTO = 0,
   /* one launch of the fused RHS + RK stage kernel per stage, replayed from CUDA graphs of
    * eight RK steps */
@@ -197,7 +198,10 @@ int weno_theta_step_batched(const wt_problem* prob, const wt_segment* segs, int3
  *   u0      [nprob][3][n] initial states (host or device)
  *   dJ_duT  [nprob][3][n] gradient of J with respect to u(T)
  *   dJ_du0  [nprob][3][n] out: gradient with respect to u(0)
- *   uT      [nprob][3][n] out (may be NULL): u(T)
+ *   uT      [nprob][3][n] out (may be NULL): u(T), bit for bit as the step entry points return it.  In
+ *           WT_MODE_FAST those evaluate smooth interfaces without the characteristic projections
+ *           (to rounding the same flux), which the differentiated pass keeps: asking for uT
+ *           then runs the steps once more
  * prob->flux must be WT_FLUX_EULER1D.  ws must hold wt_adjoint_workspace_bytes(...) bytes.
  * The environment variable WT_ADJ_TILE (31, 2031, 63, 1063 or 2063: cells per reverse tile +
  * 1000 x (items per thread - 1)) overrides the reverse kernel's tile; the gradients agree to

@@ -18,6 +18,8 @@ UNITS = {
     "wt_api.cu": [],
     "wt_kernels_fast.cu": [],
     "wt_kernels_strict.cu": ["-fmad=false"],
+    "wt_persist_fast.cu": [],
+    "wt_persist_strict.cu": ["-fmad=false"],
     "wt_noalloc.cu": [],
 }
 

@@ -155,8 +155,8 @@ Layout1D layout_1d(int m, long long n) {
   L.pitch = plane_pitch(n);
   const size_t plane = (size_t)m * L.pitch * sizeof(double);
   const size_t stage = (size_t)m * n * sizeof(double);
-  // the step-blocked tiles hold at least 27 cells
-  L.amb_ctas = (n + 26) / 27 < kStepBlockMaxCtas ? (n + 26) / 27 : kStepBlockMaxCtas;
+  // the step-blocked tiles hold at least 9 cells
+  L.amb_ctas = (n + 8) / 9 < kStepBlockMaxCtas ? (n + 8) / 9 : kStepBlockMaxCtas;
   size_t o = 0;
   L.ctl = o;
   o = align_up(o + sizeof(Ctl));
@@ -914,14 +914,14 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   //   all tiles co-resident: the persistent kernel with a halo exchange per stage;
   //   otherwise: CUDA graphs of the three stage kernels of an RK step.
   const bool strict = prob->mode == WT_MODE_STRICT;
-  const int tsb = stepblock1d_tile(prob->flux);
-  const long long nsb = (n + tsb - 1) / tsb;
   int nsm = 0;
   WT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const int tsb = stepblock1d_tile(prob->flux, n, nsm);
+  const long long nsb = (n + tsb - 1) / tsb;
   const long long ntiles = (n + tile - 1) / tile;
   int kind = 0, pgrid = 0;
   if (max_steps > 0 && prob->launch == WT_LAUNCH_AUTO) {
-    const int cap_sb = strict ? stepblock1d_capacity_strict(prob->flux) : stepblock1d_capacity_fast(prob->flux);
+    const int cap_sb = strict ? stepblock1d_capacity_strict(prob->flux, tsb) : stepblock1d_capacity_fast(prob->flux, tsb);
     if (nsb <= nsm && nsb <= cap_sb && nsb <= lay.amb_ctas) {
       kind = 2;
       pgrid = (int)nsb;
@@ -952,8 +952,8 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
         WT_CUDA(cudaMemsetAsync(amb, 0, (size_t)stepblock_mailbox_words(pgrid) * sizeof(unsigned long long), st));
         WT_CUDA(cudaMemsetAsync(U1, 0, (size_t)m * lay.pitch * sizeof(double), st));
         WT_CUDA(cudaMemsetAsync(U2, 0, (size_t)m * lay.pitch * sizeof(double), st));
-        WT_CUDA(strict ? launch_stepblock1d_strict(prob->flux, pa, pgrid, st)
-                       : launch_stepblock1d_fast(prob->flux, pa, pgrid, st));
+        WT_CUDA(strict ? launch_stepblock1d_strict(prob->flux, tsb, pa, pgrid, st)
+                       : launch_stepblock1d_fast(prob->flux, tsb, pa, pgrid, st));
       } else {
         WT_CUDA(strict ? launch_persist1d_strict(prob->flux, tile, pa, pgrid, st)
                        : launch_persist1d_fast(prob->flux, tile, pa, pgrid, st));
@@ -1523,9 +1523,9 @@ int weno_theta_adjoint(const wt_problem* prob, const wt_grid* grid, int32_t npro
   };
   const int nf = (int)tf.size(), nr = (int)tr.size();
   (void)nr;
-  // the forward stages: 127-cell tiles with six (interface, field) items per thread, the
-  // batched autotuner's pick on large Euler batches (every tile code gives the same bits)
-  constexpr int kFwdTile = 5127;
+  // the forward stages of the reverse sweep: 127-cell tiles with six (interface, field) items per
+  // thread, every reconstruction projected (its branches are recorded and differentiated)
+  constexpr int kFwdTile = kTileAdjForward;
   const int grid_f = batched_grid_size(prob, kFwdTile, nf, dev);
   auto launch_rec_stage = [&](int stage, const BatchArgs& b) {
     return strict ? launch_stage1d_batched_record_strict(stage, b, grid_f, st)
@@ -1569,14 +1569,31 @@ int weno_theta_adjoint(const wt_problem* prob, const wt_grid* grid, int32_t npro
       if ((rc = record_segment(n_steps - last0, Un)) != WT_OK) return rc;
     }
   }
-  {
+  auto check_forward = [&]() -> int {
     std::vector<Ctl> back(nprob);
     WT_CUDA(cudaMemcpyAsync(back.data(), ctl, sizeof(Ctl) * nprob, cudaMemcpyDeviceToHost, st));
     WT_CUDA(cudaStreamSynchronize(st));
     for (int p = 0; p < nprob; ++p)
       if (back[p].status != 0) return fail(back[p].status, "problem %d: forward pass reported status %d", p, back[p].status);
-  }
+    return WT_OK;
+  };
+  if ((rc = check_forward()) != WT_OK) return rc;
   if (uT) {
+    if (!strict) {
+      // u(T) bit for bit as the step entry points return it: their kernels evaluate the fluxes that
+      // the central screen proves without projections, so the pass above differs from them by rounding
+      constexpr int kStepTile = 5127;
+      WT_CUDA(launch_pack1d_batched(src, n, Un, P, dsegs, nprob, n, 3, 1, st));
+      if ((rc = init_ctl(Un)) != WT_OK) return rc;
+      BatchArgs a3[3] = {bargs(Un, nullptr, U1, tiles_f, nf), bargs(U1, Un, U2, tiles_f, nf), bargs(U2, Un, Un, tiles_f, nf)};
+      if (n_steps > 0) {
+        cudaGraphExec_t exec = nullptr;
+        if ((rc = get_batched_graph(prob, dev, kStepTile, batched_grid_size(prob, kStepTile, nf, dev), a3, &exec)) != WT_OK)
+          return rc;
+        for (int64_t step = 0; step < n_steps; ++step) WT_CUDA(cudaGraphLaunch(exec, st));
+      }
+      if ((rc = check_forward()) != WT_OK) return rc;
+    }
     if (t_dev) {
       WT_CUDA(launch_unpack1d_batched(Un, P, uT, n, dsegs, nprob, n, 3, st));
     } else {

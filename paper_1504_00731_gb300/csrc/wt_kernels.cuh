@@ -5,6 +5,9 @@
 //   stage1d     fused RHS + RK stage over a tile staged in shared memory by bulk copies
 #pragma once
 
+#include <type_traits>
+
+#include "wt_central.cuh"
 #include "wt_device.cuh"
 #include "wt_launch.h"
 
@@ -66,9 +69,74 @@ struct Tile1D {
   static constexpr size_t bytes = sizeof(double) * kTotal;
 };
 
+enum { kStage = 0, kResident = 1, kStepBlocked = 2 };  // how a tile sits in its kernel (below)
+
+// Tile of the central screen (wt_central.cuh; the fast policy's 1D Euler tiles): T cells, NT_
+// threads.  FC interfaces of the FP64 path are taken at a time, in the buffer of the difference
+// pairs (dead once the screen is done), so the tile needs no eigenvector or reconstruction
+// buffer per interface.
+template <int T, int NT_, int MODE, int IPT = 1>
+struct TileC {
+  static constexpr int M = 3;
+  static constexpr int W = (T + 9) & ~1;
+  static constexpr int NI = T + 1;
+  static constexpr int NT = NT_;
+  static constexpr bool kThree = IPT == 1;  // three threads per interface (latency-bound tiles)
+  static constexpr int FC = kThree ? (NI < 64 ? NI : 64) : (NI < 32 ? NI : 32);
+  static constexpr int kBar = 0;
+  static constexpr int kUin = 2;
+  static constexpr int kUn = kUin + 3 * W;  // u^n, kept on chip by the persistent kernels only
+  static constexpr int kF = kUn + (MODE == kStage ? 0 : 3 * W);
+  static constexpr int kVel = kF + 3 * W;
+  static constexpr int kH = kVel + W;
+  static constexpr int kSr = kH + W;        // sqrt(rho): step-blocked tiles only
+  static constexpr int kD = kSr + (MODE == kStepBlocked ? W : 0);  // [6][W] f_{k+1} - f_k, then u_{k+1} - u_k
+  static constexpr int kPair = kD + 6 * W;  // [6][W] the differences as FP32 pairs
+  // FP64 path: [9][FC], then [3][FC], [6][FC], over the pairs; after them in the step-blocked tiles,
+  // whose Roe averages are taken while the screen runs
+  static constexpr int kL = kPair + (MODE == kStepBlocked ? 6 * W : 0);
+  static constexpr int kPairN = (MODE == kStepBlocked || 18 * FC > 6 * W) ? kL - kPair + 18 * FC : 6 * W;
+  static constexpr int kRs = kL + 9 * FC;
+  static constexpr int kFs = kRs + 3 * FC;
+  static constexpr int kHf = kPair + kPairN + (kPairN & 1);  // [3][NI] interface fluxes
+  static constexpr int kRed = kHf + 3 * NI;
+  static constexpr int kQn = kRed + 4 * 32;     // ints: queue length, flag of the kernel, listed interfaces
+  static constexpr int kList = kQn + 2;         // ints [NI]: interfaces of the FP64 path; ints [NI]: marks
+  static constexpr int kQ = (kList + NI + 1) & ~1;
+  // queue of the FP64 path's unfinished reconstructions; before it, the high differences of a
+  // screen spread over three threads per interface (float4 [6][NI])
+  static constexpr int REC = kThree ? 15 : 9;
+  static constexpr int QCAP = kThree ? 96 : 64;
+  static constexpr int kQi = kQ + REC * QCAP;
+  static constexpr int kQN = REC * QCAP + QCAP / 2;
+  static constexpr int kTotal = kQ + (kThree && 12 * NI > kQN ? 12 * NI : kQN);
+  static constexpr size_t bytes = sizeof(double) * kTotal;
+};
+
+// What a stage kernel computes the interface fluxes for.  The adjoint's own forward pass keeps every
+// reconstruction projected (its branches are recorded and differentiated); kAdjRecord also
+// writes the records.
+enum { kForward = 0, kAdjForward = 1, kAdjRecord = 2 };
+template <class MATH, int FLUX, int USE>
+constexpr bool kCentralTile = MATH::kCentral && FLUX == WT_FLUX_EULER1D && USE == kForward;
+
 // the tile of a policy and flux: differences first where the policy takes them (1D Euler)
 template <class MATH, int FLUX, int T, int SPLIT = 1, int IPT = 1, bool LATE = false>
 using TileOf = Tile1D<T, FluxM<FLUX>::m, SPLIT, IPT, LATE, MATH::kDiffProj && FLUX == WT_FLUX_EULER1D>;
+
+// the tile of a kernel: mode, and (stage kernels) items per thread and use
+template <class MATH, int FLUX, int T, int MODE, int IPT = 1, int USE = kForward>
+using KernelTile = std::conditional_t<
+    kCentralTile<MATH, FLUX, USE>,
+    TileC<T,
+          // step-blocked: a thread per (interface, field, side), and a warp each for the wave speeds and
+          // per 32 Roe averages beside the screen's
+          MODE == kStepBlocked ? ((6 * (T + 1) + 31) / 32 > (3 * (T + 1) + 31) / 32 + (T + 32) / 32 + 1
+                                      ? (6 * (T + 1) + 31) / 32 * 32
+                                      : ((3 * (T + 1) + 31) / 32 + (T + 32) / 32 + 1) * 32)
+                               : Tile1D<T, FluxM<FLUX>::m, 1, IPT, MODE == kStage>::NT,
+          MODE, IPT>,
+    TileOf<MATH, FLUX, T, MODE == kStepBlocked ? 2 : 1, IPT, MODE == kStage>>;
 
 // ---------------------------------------------------------------------------------------
 // Boundary fill: copies the caller's state into the padded layout and writes the ghost
@@ -157,8 +225,6 @@ __global__ void __launch_bounds__(256) alpha1d_batched_kernel(const double* __re
 //                 three stages of an RK step need no halo exchange: the computed range shrinks
 //                 by 3 cells per side per stage, only the tile's own cells contribute to the
 //                 alphas, and only the last stage writes global memory
-enum { kStage = 0, kResident = 1, kStepBlocked = 2 };
-
 // Gathers the alpha mailbox words of `ncta` CTAs from one stage slot (4 words per CTA) with a
 // bounded wait (`limit` SM clocks) until every word carries the parity bit `pbit`; called by a
 // whole warp.  Lane l takes CTAs l, l + 32, ...; a CTA's four words are one 32-byte load
@@ -242,6 +308,493 @@ struct AlphaWait {
   unsigned int tag;
 };
 
+// ---- pieces of the central tiles (sm: the tile's shared memory, layout TileC)
+// difference k of component c (f: 0..2, u: 3..5), in FP64 and as an FP32 pair
+template <class TL>
+__device__ __forceinline__ void central_diff(double* sm, int off, int c, int k) {
+  const double* x = sm + (c < 3 ? TL::kF + c * TL::W : TL::kUin + (c - 3) * TL::W + off) + k;
+  const double d = __dsub_rn(x[1], x[0]);
+  sm[TL::kD + c * TL::W + k] = d;
+  reinterpret_cast<float2*>(sm + TL::kPair)[c * TL::W + k] = f32_pair(d);
+}
+// the high differences of component e of f and of u over the stencil of interface i, for central_project
+template <class TL>
+__device__ __forceinline__ void central_high(double* sm, int e, int i) {
+  const float2* s_pair = reinterpret_cast<const float2*>(sm + TL::kPair);
+  float4* s_x = reinterpret_cast<float4*>(sm + TL::kQ);  // [6][NI]
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    float2 d[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) d[k] = s_pair[(3 * x + e) * TL::W + i + k];
+    s_x[(3 * x + e) * TL::NI + i] = high_differences(d);
+  }
+}
+// one field's projections of an interface, taken before the alphas are known (central_project)
+struct Screen32 {
+  Roe32 r;
+  float fa[9], fb[9], ea[5], eb[5];
+  __device__ __forceinline__ bool prove(int s, const double (&alpha)[3], float eps, float aR) const {
+    const float al = f32_trunc(s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[2])), kap = s == 1 ? 2.0f : 4.0f;
+    return r.ok && prove_field(fa, fb, ea, eb, al, fmul(eps, kap * kap), aR, fmul(r.thr, kap));
+  }
+};
+template <class TL>
+__device__ __forceinline__ Roe32 central_roe32(const double* sm, int off, int i, float gm1) {
+  const double* U = sm + TL::kUin + off + i + 2;
+  const double* v = sm + TL::kVel + i + 2;
+  const double* H = sm + TL::kH + i + 2;
+  return roe32(U[0], v[0], H[0], U[1], v[1], H[1], gm1);
+}
+template <class TL>
+__device__ __forceinline__ void central_project(const double* sm, int off, int s, int i, float gm1, Screen32& z) {
+  const float2* s_pair = reinterpret_cast<const float2*>(sm + TL::kPair);
+  const float4* s_x = reinterpret_cast<const float4*>(sm + TL::kQ);
+  z.r = central_roe32<TL>(sm, off, i, gm1);
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    float d[3][5];
+    float4 h[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) d[c][k] = s_pair[(3 * x + c) * TL::W + i + k].x;
+      h[c] = s_x[(3 * x + c) * TL::NI + i];
+    }
+    Proj32 p;
+    project_stencil(z.r, d, h, p);
+    take_field(s, z.r, p, x ? z.fb : z.fa, x ? z.eb : z.ea);
+  }
+}
+// component c of C f at interface i
+template <class TL>
+__device__ __forceinline__ double central_flux(const double* sm, int c, int i) {
+  const double* d = sm + TL::kD + c * TL::W + i;
+  const double* f = sm + TL::kF + c * TL::W + i;
+  return central_value(f[2], f[3], d[0], d[1], d[3], d[4]);
+}
+// FP64 path: Roe average and eigenvectors of interface i into slot q
+template <class MATH, class TL>
+__device__ __forceinline__ void central_roe(const Stage1DArgs& a, double* sm, int off, int i, int q) {
+  const double *r = sm + TL::kUin + off + i + 2, *v = sm + TL::kVel + i + 2, *H = sm + TL::kH + i + 2;
+  double L[9], rs[3];
+  double sa, sb;
+  if constexpr (TL::kD != TL::kSr) {  // taken per cell in phase B
+    sa = sm[TL::kSr + i + 2];
+    sb = sm[TL::kSr + i + 3];
+  } else {
+    sa = MATH::sqrt_rho(r[0]);
+    sb = MATH::sqrt_rho(r[1]);
+  }
+  MATH::roe(sa, v[0], H[0], sb, v[1], H[1], a.gamma, L, rs);
+#pragma unroll
+  for (int e = 0; e < 9; ++e) sm[TL::kL + e * TL::FC + q] = L[e];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) sm[TL::kRs + e * TL::FC + q] = rs[e];
+}
+// (l.f, l.u) of cell k, and of the differences k
+template <class MATH, class TL>
+__device__ __forceinline__ void central_cell(const double* sm, int off, const double* l, int k, double& x, double& y) {
+  constexpr int W = TL::W;
+  const double *F = sm + TL::kF + k, *V = sm + TL::kUin + off + k;
+  const double f[3] = {F[0], F[W], F[2 * W]}, U[3] = {V[0], V[W], V[2 * W]};
+  MATH::project3_ab(l, f, U, x, y);
+}
+template <class MATH, class TL>
+__device__ __forceinline__ void central_dcell(const double* sm, const double* l, int k, double& x, double& y) {
+  constexpr int W = TL::W;
+  const double* D = sm + TL::kD + k;
+  const double f[3] = {D[0], D[W], D[2 * W]}, U[3] = {D[3 * W], D[4 * W], D[5 * W]};
+  MATH::project3_ab(l, f, U, x, y);
+}
+// component c of h from the reconstructions of slot q
+template <class MATH, class TL>
+__device__ __forceinline__ double central_back(const double* sm, int c, int q) {
+  constexpr int FC = TL::FC;
+  const double *r = sm + TL::kRs + q, *F = sm + TL::kFs + q;
+  const double rs[3] = {r[0], r[FC], r[2 * FC]};
+  const double Fs[3] = {F[0] + F[3 * FC], F[FC] + F[4 * FC], F[2 * FC] + F[5 * FC]};
+  return MATH::backproject_c(c, rs, Fs);
+}
+
+// FP64 path of the latency-bound tiles: two adjacent threads per (interface, field), one per side.
+// Each takes the products of its centre cell and of its outer two differences (0, 1 or 4, 3) and the
+// pair swaps them (whole warps).  The - side reconstructs its stencil negated: the reconstruction is
+// odd in its data bit for bit (squares and comparisons do not see the sign, every other step is
+// a rounded linear operation), so no selects or negations of the differences are needed.
+template <class MATH, class TL>
+struct SidePair {
+  double o[6], p[6];
+  __device__ __forceinline__ void project(const double* sm, int off, bool has, int s, int i, int q) {
+    constexpr int FC = TL::FC;
+    const int side = threadIdx.x & 1;
+#pragma unroll
+    for (int z = 0; z < 6; ++z) o[z] = 0.0;
+    if (has) {
+      const double* L = sm + TL::kL + 3 * s * FC + q;
+      const double l[3] = {L[0], L[FC], L[2 * FC]};
+      central_cell<MATH, TL>(sm, off, l, i + 2 + side, o[0], o[1]);
+      central_dcell<MATH, TL>(sm, l, side ? i + 4 : i, o[2], o[3]);
+      central_dcell<MATH, TL>(sm, l, side ? i + 3 : i + 1, o[4], o[5]);
+    }
+#pragma unroll
+    for (int z = 0; z < 6; ++z) p[z] = __shfl_xor_sync(0xffffffffu, o[z], 1);
+  }
+  // the side's reconstruction into F, or a record for central_deferred
+  __device__ __forceinline__ void reconstruct(const Stage1DArgs& a, double* sm, const double (&alpha)[3], int s, int q,
+                                              bool proven) const {
+    int* s_cnt = reinterpret_cast<int*>(sm + TL::kQn);
+    const int side = threadIdx.x & 1;
+    const unsigned long long sg = side ? 0x8000000000000000ull : 0ull;
+    // the side's stencil order: its own differences 0, 1 (or 4, 3), its partner's in reverse, the
+    // middle one from the centres
+    const double da[5] = {o[2], o[4], flip_sign(p[0] - o[0], sg), p[4], p[2]};
+    const double db[5] = {o[3], o[5], flip_sign(p[1] - o[1], sg), p[5], p[3]};
+    const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[2]);
+    const double sa = flip_sign(al, sg);
+    double d[5], rec[TL::REC];
+#pragma unroll
+    for (int z = 0; z < 5; ++z) d[z] = fma(sa, db[z], da[z]);
+    const double q2 = fma(al, o[1], flip_sign(o[0], sg));  // + side: a2 + alpha b2; - side: alpha b3 - a3
+    const int dst = (3 * side + s) * TL::FC + q;
+    double* s_F = sm + TL::kFs;
+    // a proven field is restricted on both sides with theta = 0 (or of no matter)
+    const int scr = proven ? 2 : MATH::weno_front_d(d, q2, a.eps, a.alpha_R, rec);
+    if (scr != 0) {
+      s_F[dst] = flip_sign(MATH::linear_theta(d[0], d[1], d[2], d[3], d[4], q2, scr == 1), sg);
+      return;
+    }
+    const int slot = atomicAdd(&s_cnt[0], 1);
+    if (slot < TL::QCAP) {
+#pragma unroll
+      for (int z = 0; z < TL::REC; ++z) sm[TL::kQ + z * TL::QCAP + slot] = rec[z];
+      reinterpret_cast<int*>(sm + TL::kQi)[slot] = dst | (side ? (1 << 30) : 0);
+    } else {
+      s_F[dst] = flip_sign(MATH::weno_d(d, q2, a.eps, a.alpha_R), sg);
+    }
+  }
+};
+// a quad of lanes per deferred stencil (FastMath::weno_back_quad)
+template <class MATH, class TL>
+__device__ __forceinline__ void central_deferred(const Stage1DArgs& a, double* sm) {
+  const int nq = min(*reinterpret_cast<const int*>(sm + TL::kQn), TL::QCAP);
+  for (int b0 = 0; b0 < nq; b0 += TL::NT / 4) {
+    const int t = b0 + ((int)threadIdx.x >> 2), z = threadIdx.x & 3;
+    if (t < nq) {  // the same for the four lanes of a quad
+      double rec[TL::REC];
+#pragma unroll
+      for (int y = 0; y < TL::REC; ++y) rec[y] = sm[TL::kQ + y * TL::QCAP + t];
+      const double out = MATH::weno_back_quad(z, rec, a.eps, a.alpha_R, 0xfu << (threadIdx.x & 28));
+      const int qi = reinterpret_cast<const int*>(sm + TL::kQi)[t];
+      if (z == 0)
+        sm[TL::kFs + (qi & ((1 << 30) - 1))] = flip_sign(out, (qi >> 30) & 1 ? 0x8000000000000000ull : 0ull);
+    }
+  }
+}
+
+// Step-blocked tiles: the chain of the CTA whose tile holds a shock, for which all others wait at the
+// next alpha exchange, is what a stage lasts.  The screen's differences and projections run on the
+// first warps, the FP64 Roe average of every interface on two others (2.2k clocks longer than
+// the screen), the wave speeds and the alpha exchange on the last; the screen's warps decide
+// the fields as soon as the alphas are in (about 4.3k clocks into the stage), still before
+// the Roe averages are.  Then the pairs of the listed interfaces go on.  Returns false as
+// stage1d_compute does.
+template <class MATH, class TL>
+__device__ __forceinline__ bool central_fluxes_blocked(const Stage1DArgs& a, const int Tc, const int off,
+                                                       double (&alpha)[3], double& dt, double* sm,
+                                                       const AlphaWait& aw) {
+  constexpr int W = TL::W, NI = TL::NI, NT = TL::NT;
+  constexpr int kSW = NT / 32 - 1;                  // the speed warp
+  constexpr int kRoeThreads = ((NI + 31) / 32) * 32;
+  constexpr int NP = NT - 32 - kRoeThreads;         // threads of the screen
+  static_assert(3 * NI <= NP && 6 * NI <= NT && TL::FC == NI, "one (interface, field) and side per thread");
+  const int tid = threadIdx.x;
+  const int ni = Tc + 1, nd = Tc + 2 * G - 1;
+  int* s_cnt = reinterpret_cast<int*>(sm + TL::kQn);
+  int* s_mark = reinterpret_cast<int*>(sm + TL::kList) + NI;
+  double* s_dt = sm + TL::kRed + 4;  // beside the alphas
+  const unsigned long long* s_alpha = reinterpret_cast<const unsigned long long*>(sm + TL::kRed);
+  const bool has = tid < 3 * ni;  // (within the screen's threads)
+  const int s = has ? tid / ni : 0, i = has ? tid - s * ni : 0;
+  if (tid < NP) {
+    for (int idx = tid; idx < 6 * W; idx += NP) {
+      const int c = idx / W, k = idx - c * W;
+      if (k < nd) central_diff<TL>(sm, off, c, k);
+    }
+    if (tid < NI) s_mark[tid] = 0;
+    named_barrier_sync(2, NP);
+    if (has) central_high<TL>(sm, s, i);
+    named_barrier_sync(2, NP);
+    const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
+    Screen32 z;
+    if (has) {
+      central_project<TL>(sm, off, s, i, gm1, z);
+      sm[TL::kHf + s * NI + i] = central_flux<TL>(sm, s, i);
+    }
+    named_barrier_sync(4, NP + 32);  // the speed warp holds the alphas of every CTA
+#pragma unroll
+    for (int f = 0; f < 3; ++f) alpha[f] = bits_to_double(s_alpha[f]);
+    if (has && !(fmul(aR, eps) > 1e-30f && z.prove(s, alpha, eps, aR))) atomicOr(&s_mark[i], 1 << s);
+  } else if ((tid >> 5) != kSW) {
+    if (tid - NP < ni) central_roe<MATH, TL>(a, sm, off, tid - NP, tid - NP);
+  } else {
+    __syncwarp();
+    named_barrier_arrive(4, NP + 32);
+    if (aw.first_stage) {  // one warp takes the step (an FP64 division)
+      const double a0 = bits_to_double(s_alpha[0]), a2 = bits_to_double(s_alpha[2]);
+      double h = aw.dt_fixed > 0.0 ? aw.dt_fixed : MATH::cfl_dt(aw.cfl, a.dx, (a0 < a2) ? a2 : a0);
+      const double rem = aw.t_final - aw.t;
+      if (rem < h) h = rem;
+      if ((tid & 31) == 0) {
+        *s_dt = h;
+        if (aw.clear >= 0 && s_cnt[1] == 1) a.ctl->dt = h;
+      }
+    }
+  }
+  __syncthreads();
+  if (s_cnt[1] != 1) return false;
+#pragma unroll
+  for (int f = 0; f < 3; ++f) alpha[f] = bits_to_double(s_alpha[f]);
+  if (aw.first_stage) dt = *s_dt;
+  {  // the pair of threads of (interface, field) it = tid / 2
+    const int it = tid >> 1;
+    const bool phas = it < 3 * ni;
+    const int ps = phas ? it / ni : 0, pi = phas ? it - ps * ni : 0;
+    const int m = phas ? s_mark[pi] : 0;
+    if (__any_sync(0xffffffffu, m != 0)) {
+      SidePair<MATH, TL> pair;
+      pair.project(sm, off, m != 0, ps, pi, pi);
+      if (m != 0) pair.reconstruct(a, sm, alpha, ps, pi, !((m >> ps) & 1));
+    }
+  }
+  __syncthreads();
+  if (s_cnt[0] > 0) {  // the same for every thread
+    central_deferred<MATH, TL>(a, sm);
+    __syncthreads();
+  }
+  if (has && s_mark[i] != 0) sm[TL::kHf + s * NI + i] = central_back<MATH, TL>(sm, s, i);
+  __syncthreads();
+  return true;
+}
+
+// Interface fluxes of a tile by the central screen (wt_central.cuh), in place of phases C0, C1 and D:
+//   D1  differences of f and u between neighbouring cells, in FP64 and as FP32 pairs
+//   D2  per interface, the screen: the interface takes C f (central_value), or is listed (with the
+//       fields that are not proven in the high half) for
+//   D3  the FP64 path, FC listed interfaces at a time: Roe average, projections, both
+//       reconstructions of each field, back-projection
+// Throughput tiles (IPT > 1) give an interface's screen to one thread (about 1400 FP32 and integer
+// instructions, no redundant ones).  The others (IPT = 1: latency-bound, three threads or more
+// per interface) give each thread one field, and one component of the high differences,
+// exchanged through shared memory.
+template <class MATH, class TL>
+__device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int Tc, const int off,
+                                               const double (&alpha)[3], double* sm) {
+  constexpr int W = TL::W, NI = TL::NI, NT = TL::NT, FC = TL::FC, QCAP = TL::QCAP;
+  constexpr bool kThree = TL::kThree;
+  static_assert(!kThree || 3 * NI <= NT, "one (interface, field) per thread");
+  double* s_uin = sm + TL::kUin;
+  double* s_f = sm + TL::kF;
+  double* s_vel = sm + TL::kVel;
+  double* s_H = sm + TL::kH;
+  double* s_d = sm + TL::kD;
+  float2* s_pair = reinterpret_cast<float2*>(sm + TL::kPair);
+  double* s_h = sm + TL::kHf;
+  double* s_L = sm + TL::kL;
+  double* s_rs = sm + TL::kRs;
+  double* s_F = sm + TL::kFs;  // [2 sides * 3 fields][FC]
+  double* s_q = sm + TL::kQ;
+  int* s_qi = reinterpret_cast<int*>(sm + TL::kQi);
+  int* s_cnt = reinterpret_cast<int*>(sm + TL::kQn);  // [0] queue length, [2] listed interfaces
+  int* s_list = reinterpret_cast<int*>(sm + TL::kList);
+  int* s_mark = s_list + NI;
+  const int tid = threadIdx.x;
+  const int ni = Tc + 1, nd = Tc + 2 * G - 1;
+  auto take_diff = [&](const int c, const int k) { central_diff<TL>(sm, off, c, k); };
+
+  // ---- D1
+  if (kThree) {
+    for (int idx = tid; idx < 6 * W; idx += NT) {
+      const int c = idx / W, k = idx - c * W;
+      if (k < nd) take_diff(c, k);
+    }
+    for (int i = tid; i < NI; i += NT) s_mark[i] = 0;
+  } else {
+    for (int k = tid; k < nd; k += NT) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) take_diff(c, k);
+    }
+  }
+  __syncthreads();
+
+  // ---- D2
+  const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
+  const bool screenable = fmul(aR, eps) > 1e-30f;
+  auto central = [&](const int c, const int i) { s_h[c * NI + i] = central_flux<TL>(sm, c, i); };
+  if constexpr (kThree) {
+    const bool has = tid < 3 * ni;
+    const int s = has ? tid / ni : 0, i = has ? tid - s * ni : 0;
+    if (has) central_high<TL>(sm, s, i);
+    __syncthreads();
+    if (has) {
+      Screen32 z;
+      central_project<TL>(sm, off, s, i, gm1, z);
+      if (!(screenable && z.prove(s, alpha, eps, aR))) atomicOr(&s_mark[i], 1 << s);
+    }
+    __syncthreads();
+    // the list (a warp per 32 interfaces), and C f of the others
+    for (int w = tid >> 5; w * 32 < ni; w += NT / 32) {
+      int at = 0;
+      for (int v = 0; v < w; ++v) at += __popc(__ballot_sync(0xffffffffu, s_mark[32 * v + (tid & 31)] != 0));
+      const int q = 32 * w + (tid & 31);
+      const bool m = q < ni && s_mark[q] != 0;
+      const unsigned b = __ballot_sync(0xffffffffu, m);
+      if (m) s_list[at + __popc(b & ((1u << (tid & 31)) - 1u))] = q | (s_mark[q] << 16);
+      if ((w + 1) * 32 >= ni && (tid & 31) == 0) s_cnt[2] = at + __popc(b);
+    }
+    for (int idx = tid; idx < 3 * NI; idx += NT) {
+      const int c = idx / NI, q = idx - c * NI;
+      if (q < ni && s_mark[q] == 0) central(c, q);
+    }
+  } else {
+    for (int i = tid; i < ni; i += NT) {
+      const Roe32 r = roe32(s_uin[off + i + 2], s_vel[i + 2], s_H[i + 2], s_uin[off + i + 3], s_vel[i + 3], s_H[i + 3],
+                            gm1);
+      Proj32 pf, pu;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        float d[3][5];
+        float4 h[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          float2 q[5];
+#pragma unroll
+          for (int k = 0; k < 5; ++k) {
+            q[k] = s_pair[(3 * x + c) * W + i + k];
+            d[c][k] = q[k].x;
+          }
+          h[c] = high_differences(q);
+        }
+        project_stencil(r, d, h, x ? pu : pf);
+      }
+      int bad = 0;  // bit s: field s is not proven
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        float fa[9], fb[9], ea[5], eb[5];
+        take_field(s, r, pf, fa, ea);
+        take_field(s, r, pu, fb, eb);
+        const float kap = s == 1 ? 2.0f : 4.0f;
+        if (!(prove_field(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(r.thr, kap)) && r.ok &&
+              screenable))
+          bad |= 1 << s;
+      }
+      if (bad == 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) central(c, i);
+      } else {
+        s_list[atomicAdd(&s_cnt[2], 1)] = i | (bad << 16);
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- D3
+  const int nl = s_cnt[2];
+  for (int base = 0; base < nl; base += FC) {
+    const int nc = min(nl - base, FC);
+    for (int q = tid; q < nc; q += NT) central_roe<MATH, TL>(a, sm, off, s_list[base + q] & 0xffff, q);
+    __syncthreads();
+    auto proj_cell = [&](const double* l, const int k, double& x, double& y) { central_cell<MATH, TL>(sm, off, l, k, x, y); };
+    auto proj_diff = [&](const double* l, const int k, double& x, double& y) { central_dcell<MATH, TL>(sm, l, k, x, y); };
+    if constexpr (kThree) {
+      // two adjacent threads per (interface, field), one per side (SidePair)
+      for (int w0 = (tid >> 5) * 32; w0 < 6 * nc; w0 += NT) {  // warp-uniform
+        const int it = (w0 + (tid & 31)) >> 1;
+        const bool has = it < 3 * nc;
+        const int s = has ? it / nc : 0, q = it - s * nc;
+        SidePair<MATH, TL> p;
+        const int e = has ? s_list[base + q] : 0;
+        p.project(sm, off, has, s, e & 0xffff, q);
+        if (has) p.reconstruct(a, sm, alpha, s, q, !((e >> (16 + s)) & 1));
+      }
+      __syncthreads();
+      central_deferred<MATH, TL>(a, sm);
+      __syncthreads();
+      // one component of h per thread
+      for (int idx = tid; idx < 3 * nc; idx += NT) {
+        const int c = idx / nc, q = idx - c * nc;
+        s_h[c * NI + (s_list[base + q] & 0xffff)] = central_back<MATH, TL>(sm, c, q);
+      }
+    } else {
+      for (int it = tid; it < 3 * nc; it += NT) {
+        const int s = it / nc, q = it - s * nc, i = s_list[base + q] & 0xffff;
+        const bool proven = !((s_list[base + q] >> (16 + s)) & 1);
+        const double l[3] = {s_L[(3 * s) * FC + q], s_L[(3 * s + 1) * FC + q], s_L[(3 * s + 2) * FC + q]};
+        double da[5], db[5], a2, b2, a3, b3;
+        proj_cell(l, i + 2, a2, b2);
+        proj_cell(l, i + 3, a3, b3);
+        proj_diff(l, i, da[0], db[0]);
+        proj_diff(l, i + 1, da[1], db[1]);
+        proj_diff(l, i + 3, da[3], db[3]);
+        proj_diff(l, i + 4, da[4], db[4]);
+        da[2] = a3 - a2;
+        db[2] = b3 - b2;
+        const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[2]);
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          double d[5], q2, out;
+          MATH::side_diffs(da, db, a2, b2, a3, b3, al, side != 0, d, q2);
+          const int dst = (3 * side + s) * FC + q;
+          typename MATH::WenoPart w;
+          if (proven) {
+            s_F[dst] = MATH::linear_theta(d[0], d[1], d[2], d[3], d[4], q2, false);
+          } else if (MATH::weno_begin_d(d, q2, a.eps, a.alpha_R, out, w)) {
+            s_F[dst] = out;
+          } else {
+            // the nonlinear weights go to a second pass over full warps
+            const int slot = atomicAdd(&s_cnt[0], 1);
+            if (slot < QCAP) {
+#pragma unroll
+              for (int z = 0; z < 4; ++z) s_q[z * QCAP + slot] = w.e[z];
+              s_q[4 * QCAP + slot] = w.tau;
+#pragma unroll
+              for (int z = 0; z < 4; ++z) s_q[(5 + z) * QCAP + slot] = w.fh[z];
+              s_qi[slot] = dst | (w.theta1 ? (1 << 30) : 0);
+            } else {
+              s_F[dst] = MATH::weno_finish(w);
+            }
+          }
+        }
+      }
+      __syncthreads();
+      const int nq = min(s_cnt[0], QCAP);
+      for (int t = tid; t < nq; t += NT) {
+        typename MATH::WenoPart w;
+#pragma unroll
+        for (int z = 0; z < 4; ++z) w.e[z] = s_q[z * QCAP + t];
+        w.tau = s_q[4 * QCAP + t];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) w.fh[z] = s_q[(5 + z) * QCAP + t];
+        const int qi = s_qi[t];
+        w.theta1 = (qi >> 30) & 1;
+        s_F[qi & ((1 << 30) - 1)] = MATH::weno_finish(w);
+      }
+      __syncthreads();
+      for (int q = tid; q < nc; q += NT) {
+        const int i = s_list[base + q] & 0xffff;
+        const double rs[3] = {s_rs[q], s_rs[FC + q], s_rs[2 * FC + q]};
+        const double F[3] = {s_F[q] + s_F[3 * FC + q], s_F[FC + q] + s_F[4 * FC + q], s_F[2 * FC + q] + s_F[5 * FC + q]};
+        double h[3];
+        MATH::backproject(rs, F, h);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) s_h[c * NI + i] = h[c];
+      }
+    }
+    if (tid == 0) s_cnt[0] = 0;
+    __syncthreads();
+  }
+}
+
 // Phases B-E of one stage over the cells [js, js + Ts) whose window [js - 3, js + Ts + 3) is
 // in shared memory at s_uin[off...] (s_un for stages 2 and 3), with the stage's dt.  The
 // wave speeds of the cells of [own_lo, own_hi) go to the alpha ring: in kStage and kResident
@@ -250,7 +803,7 @@ struct AlphaWait {
 // written and then gathered by the last warp while the others go on).  Returns false if a
 // wait for the alphas timed out (the flag word then holds 2) or, at the first stage of a
 // step-blocked RK step, if some CTA has seen a failure (flag word 3): the step is not taken.
-template <class MATH, int FLUX, int STAGE, int T, int MODE, int IPT = 1, bool REC = false>
+template <class MATH, int FLUX, int STAGE, int T, int MODE, int IPT = 1, int USE = kForward>
 __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long long js, const int Ts, const int off,
                                                 const long long own_lo, const long long own_hi,
                                                 double (&alpha)[FluxM<FLUX>::m], double& dt, double* sm,
@@ -260,9 +813,13 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   constexpr int SPLIT = (MODE == kStepBlocked) ? 2 : 1;
   static_assert(IPT == 1 || MODE != kStepBlocked, "the step-blocked tiles carry one item per thread pair");
   constexpr bool LATE = (MODE == kStage);
-  using TL = TileOf<MATH, FLUX, T, SPLIT, IPT, LATE>;
+  constexpr bool REC = USE == kAdjRecord;
+  constexpr bool CENTRAL = kCentralTile<MATH, FLUX, USE>;
+  using TL = KernelTile<MATH, FLUX, T, MODE, IPT, USE>;
   constexpr int W = TL::W, NI = TL::NI, NT = TL::NT;
-  constexpr bool DP = MATH::kDiffProj && FLUX == WT_FLUX_EULER1D;  // differences first (phase C1)
+  // differences first (phase C1): the adjoint's forward tiles (the central tiles' FP64 path does so too)
+  constexpr bool DP = MATH::kDiffProj && FLUX == WT_FLUX_EULER1D && !CENTRAL;
+  static_assert(!DP || (MODE == kStage && IPT > 1), "the adjoint's forward tiles");
   static_assert(NT * IPT >= SPLIT * M * NI, "IPT (interface, field) items per thread (one per thread pair with SPLIT = 2)");
   double* s_uin = sm + TL::kUin;
   double* s_un = sm + TL::kUn;
@@ -291,7 +848,10 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   constexpr int kSW = NT / 32 - 1;  // the speed warp (step-blocked)
   unsigned long long* s_alpha = reinterpret_cast<unsigned long long*>(s_red);
   int* s_aflag = reinterpret_cast<int*>(sm + TL::kQn) + 1;
-  if (tid == 0) *reinterpret_cast<int*>(sm + TL::kQn) = 0;
+  if (tid == 0) {
+    *reinterpret_cast<int*>(sm + TL::kQn) = 0;
+    if (CENTRAL) reinterpret_cast<int*>(sm + TL::kQn)[2] = 0;
+  }
   if (MODE == kStepBlocked && (tid >> 5) == kSW) {
     const int lane = tid & 31;
     named_barrier_arrive(1, NT);  // phase B does not wait for the speeds
@@ -359,24 +919,48 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         }
       }
       if (FLUX == WT_FLUX_EULER1D) {
-        double f[3], u, H, sr, p;
-        MATH::euler_cell(U, a.gamma, f, u, H, sr, p);
+        double f[3], u, H, sr = 0.0, p;
+        if constexpr (CENTRAL) {
+          MATH::euler_cell_flux(U, a.gamma, f, u, H);
+        } else {
+          MATH::euler_cell(U, a.gamma, f, u, H, sr, p);
+        }
         if (!finite3(U)) flag_error(ctl, WT_ERR_NONPHYSICAL);
         s_f[k] = f[0];
         s_f[W + k] = f[1];
         s_f[2 * W + k] = f[2];
         s_vel[k] = u;
         s_H[k] = H;
-        s_sr[k] = sr;
+        if constexpr (!CENTRAL) s_sr[k] = sr;
       } else {
         const double xv = U[0];
         if (!isfinite(xv)) flag_error(ctl, WT_ERR_NONPHYSICAL);
         s_f[k] = (FLUX == WT_FLUX_ADVECTION) ? MATH::flux_advection(a.adv_speed, xv) : MATH::flux_burgers(xv);
       }
     }
+    if constexpr (CENTRAL && MODE == kStepBlocked) {
+      // sqrt(rho) for the Roe warps, on two warps that hold no cell above
+      static_assert(W <= 64 && NT / 32 - 2 > 2, "two warps cover the window");
+      const int sw = tid >> 5, q = (sw == 2 ? 0 : 32) + (tid & 31);
+      if ((sw == 2 || sw == NT / 32 - 2) && q < cells) {
+        const long long x = js - G + q;
+        const bool lo_g = x < 0 && a.bc_lo != WT_BC_PERIODIC, hi_g = x >= n && a.bc_hi != WT_BC_PERIODIC;
+        const long long xs = hi_g ? (a.bc_hi == WT_BC_OUTFLOW ? n - 1 : 2 * n - 1 - x)
+                                  : (lo_g ? (a.bc_lo == WT_BC_OUTFLOW ? 0 : -1 - x) : x);
+        sm[TL::kSr + q] = MATH::sqrt_rho(s_uin[off + q + (int)(xs - x)]);
+      }
+    }
     if (MODE == kStepBlocked) named_barrier_sync(1, NT);
   }
   if (MODE != kStepBlocked) __syncthreads();
+  const double* hsrc = s_h;
+  if constexpr (CENTRAL) {
+    if constexpr (MODE == kStepBlocked) {
+      if (!central_fluxes_blocked<MATH, TL>(a, Tc, off, alpha, dt, sm, aw)) return false;
+    } else {
+      central_fluxes<MATH, TL>(a, Tc, off, alpha, sm);
+    }
+  } else {
   // step-blocked scalar fluxes have no phase C0: the alphas are awaited here
   if (MODE == kStepBlocked && FLUX != WT_FLUX_EULER1D) __syncthreads();
   // Step-blocked: where the speed warp holds no phase-C1 item (stages whose items fit in the
@@ -416,28 +1000,13 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
 #pragma unroll
       for (int e = 0; e < 3; ++e) s_rs[e * NI + i] = rs[e];
     }
-    if constexpr (DP && MODE != kStage) {
-      // differences k = i + 2 by the thread of interface i, the four outer ones (k = 0, 1,
-      // Tc + 3, Tc + 4) by the next four threads, none of them the speed warp (static_assert
-      // below)
-      const int k = tid < ni ? tid + 2 : (tid < ni + 2 ? tid - ni : Tc + 3 + (tid - ni - 2));
-      if (tid < ni + 4) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          sm[TL::kDf + c * W + k] = s_f[c * W + k + 1] - s_f[c * W + k];
-          sm[TL::kDu + c * W + k] = s_uin[c * W + off + k + 1] - s_uin[c * W + off + k];
-        }
-      }
-    }
     c0_barrier();
   }
-  static_assert(!DP || MODE == kStage || NI + 4 <= NT - (MODE == kStepBlocked ? 32 : 0),
-                "outer differences fit the C0 threads");
   // DP: the differences of f and u between neighbouring window cells (f's over the per-cell
   // Roe inputs, read for the last time in phase C0), by the threads of phase C0
   double* s_df = sm + TL::kDf;
   double* s_du = sm + TL::kDu;
-  if constexpr (DP && MODE == kStage) {
+  if constexpr (DP) {
     if (!(sw_free && (tid >> 5) == kSW)) {
       const int np = sw_free ? NT - 32 : NT;
       for (int k = tid; k < cells - 1; k += np) {
@@ -470,10 +1039,6 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   // pa, pb: (l.f, l.u) of the stencil cells i .. i + 5 (window index), in the order of the
   // side's stencil with SPLIT = 2 (the - side reads the cells mirrored, Eq. (flux_split_lf))
   double pa[6], pb[6];
-  // DP: (da_k, db_k) the products of the stencil's cell differences, (a2, b2) and (a3, b3) those
-  // of its two centre cells (MATH::side_diffs); with SPLIT = 2 the + thread takes the centre
-  // cell 2 and differences 0, 1, the - thread cell 3 and differences 4, 3, and the pair swaps them
-  double da[5], db[5], a2 = 0.0, b2 = 0.0, a3 = 0.0, b3 = 0.0;
   auto proj_cell = [&](const double* l, const int k, double& x, double& y) {
     double f[3] = {s_f[k], s_f[W + k], s_f[2 * W + k]};
     double U[3] = {s_uin[off + k], s_uin[W + off + k], s_uin[2 * W + off + k]};
@@ -484,48 +1049,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
     double U[3] = {s_du[k], s_du[W + k], s_du[2 * W + k]};
     MATH::project3_ab(l, f, U, x, y);
   };
-  if constexpr (DP && SPLIT == 2) {
-    double o[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (has_item) {
-      double l[3] = {s_L[(3 * s) * NI + i], s_L[(3 * s + 1) * NI + i], s_L[(3 * s + 2) * NI + i]};
-      proj_cell(l, i + 2 + side2, o[0], o[1]);
-      proj_diff(l, side2 ? i + 4 : i, o[2], o[3]);
-      proj_diff(l, side2 ? i + 3 : i + 1, o[4], o[5]);
-    }
-    if ((tid >> 5) * 32 < SPLIT * M * ni) {
-      double p[6];
-#pragma unroll
-      for (int r = 0; r < 6; ++r) p[r] = __shfl_xor_sync(0xffffffffu, o[r], 1);
-      // the side's stencil order: its own products are differences 0, 1 (+ side) or 4, 3
-      // (- side, mirrored), its partner's the other two in reverse, and difference 2 is
-      // a3 - a2 on both sides (the partner's centre minus its own, negated on the - side)
-      const unsigned long long sg = side2 ? 0x8000000000000000ull : 0ull;
-      da[0] = o[2];
-      db[0] = o[3];
-      da[1] = o[4];
-      db[1] = o[5];
-      da[4] = p[2];
-      db[4] = p[3];
-      da[3] = p[4];
-      db[3] = p[5];
-      da[2] = flip_sign(p[0] - o[0], sg);
-      db[2] = flip_sign(p[1] - o[1], sg);
-      a2 = o[0];  // the own centre cell's products
-      b2 = o[1];
-    }
-  } else if constexpr (DP) {
-    if (has_item && IPT == 1) {
-      double l[3] = {s_L[(3 * s) * NI + i], s_L[(3 * s + 1) * NI + i], s_L[(3 * s + 2) * NI + i]};
-      proj_cell(l, i + 2, a2, b2);
-      proj_cell(l, i + 3, a3, b3);
-      proj_diff(l, i, da[0], db[0]);
-      proj_diff(l, i + 1, da[1], db[1]);
-      proj_diff(l, i + 3, da[3], db[3]);
-      proj_diff(l, i + 4, da[4], db[4]);
-      da[2] = a3 - a2;
-      db[2] = b3 - b2;
-    }
-  } else if constexpr (SPLIT == 2) {
+  if constexpr (SPLIT == 2) {
     double oa[3] = {0.0, 0.0, 0.0}, ob[3] = {0.0, 0.0, 0.0};
     if (has_item) {
       if (FLUX == WT_FLUX_EULER1D) {
@@ -556,7 +1080,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         pb[5 - h] = __shfl_xor_sync(0xffffffffu, ob[h], 1);
       }
     }
-  } else if (has_item && IPT == 1) {
+  } else if (has_item && IPT == 1 && !DP) {
     if (FLUX == WT_FLUX_EULER1D) {
       double l[3] = {s_L[(3 * s) * NI + i], s_L[(3 * s + 1) * NI + i], s_L[(3 * s + 2) * NI + i]};
 #pragma unroll
@@ -640,86 +1164,45 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   };
   if constexpr (DP) {
     // differences first: the reconstructions from their stencils' differences and q_2
-    // (step-blocked: sg negates the result of a - side thread, which reconstructs its stencil
-    // negated; its queue record carries bit 30)
-    auto reconstruct_d = [&](const double* d, const double q2, const int dst, const unsigned long long sg = 0ull) {
+    auto reconstruct_d = [&](const double* d, const double q2, const int dst) {
       double out;
-      if constexpr (MODE == kStepBlocked) {
-        double rec[TL::REC];
-        if (MATH::weno_front_d(d, q2, a.eps, a.alpha_R, out, rec)) {
-          s_F[dst] = flip_sign(out, sg);
-        } else {
-          const int slot = atomicAdd(s_qn, 1);
-          if (slot < QCAP) {
-#pragma unroll
-            for (int r = 0; r < TL::REC; ++r) s_q[r * QCAP + slot] = rec[r];
-            s_qi[slot] = dst | (sg ? (1 << 30) : 0);
-          } else {
-            s_F[dst] = flip_sign(MATH::weno_d(d, q2, a.eps, a.alpha_R), sg);
-          }
-        }
+      typename MATH::WenoPart w;
+      if (MATH::weno_begin_d(d, q2, a.eps, a.alpha_R, out, w)) {
+        s_F[dst] = out;
+        if constexpr (REC) s_fl[dst] = (unsigned char)(1 | (w.theta1 ? 2 : 0));
       } else {
-        typename MATH::WenoPart w;
-        if (MATH::weno_begin_d(d, q2, a.eps, a.alpha_R, out, w)) {
-          s_F[dst] = out;
-          if constexpr (REC) s_fl[dst] = (unsigned char)(1 | (w.theta1 ? 2 : 0));
+        if constexpr (REC) s_fl[dst] = (unsigned char)(w.theta1 ? 2 : 0);
+        const int slot = atomicAdd(s_qn, 1);
+        if (slot < QCAP) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s_q[k * QCAP + slot] = w.e[k];
+          s_q[4 * QCAP + slot] = w.tau;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s_q[(5 + k) * QCAP + slot] = w.fh[k];
+          s_qi[slot] = dst | (w.theta1 ? (1 << 30) : 0);
         } else {
-          if constexpr (REC) s_fl[dst] = (unsigned char)(w.theta1 ? 2 : 0);
-          const int slot = atomicAdd(s_qn, 1);
-          if (slot < QCAP) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s_q[k * QCAP + slot] = w.e[k];
-            s_q[4 * QCAP + slot] = w.tau;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s_q[(5 + k) * QCAP + slot] = w.fh[k];
-            s_qi[slot] = dst | (w.theta1 ? (1 << 30) : 0);
-          } else {
-            s_F[dst] = MATH::weno_finish(w);
-          }
+          s_F[dst] = MATH::weno_finish(w);
         }
       }
     };
-    if constexpr (IPT > 1) {
-      for (int it2 = tid; it2 < M * ni; it2 += NT) {
-        const int s2 = it2 / ni, i2 = it2 - s2 * ni;
-        double l[3] = {s_L[(3 * s2) * NI + i2], s_L[(3 * s2 + 1) * NI + i2], s_L[(3 * s2 + 2) * NI + i2]};
-        double ea[5], eb[5], c2a, c2b, c3a, c3b;
-        proj_cell(l, i2 + 2, c2a, c2b);
-        proj_cell(l, i2 + 3, c3a, c3b);
-        proj_diff(l, i2, ea[0], eb[0]);
-        proj_diff(l, i2 + 1, ea[1], eb[1]);
-        proj_diff(l, i2 + 3, ea[3], eb[3]);
-        proj_diff(l, i2 + 4, ea[4], eb[4]);
-        ea[2] = c3a - c2a;
-        eb[2] = c3b - c2b;
-        const double al = (s2 == 0) ? alpha[0] : ((s2 == 1) ? alpha[1] : alpha[M - 1]);
-        double d[5], q2;
-        MATH::side_diffs(ea, eb, c2a, c2b, c3a, c3b, al, false, d, q2);
-        reconstruct_d(d, q2, s2 * NI + i2);
-        MATH::side_diffs(ea, eb, c2a, c2b, c3a, c3b, al, true, d, q2);
-        reconstruct_d(d, q2, M * NI + s2 * NI + i2);
-      }
-    } else if (has_item) {
-      const double al = (s == 0) ? alpha[0] : ((s == 1) ? alpha[1] : alpha[M - 1]);
+    for (int it2 = tid; it2 < M * ni; it2 += NT) {
+      const int s2 = it2 / ni, i2 = it2 - s2 * ni;
+      double l[3] = {s_L[(3 * s2) * NI + i2], s_L[(3 * s2 + 1) * NI + i2], s_L[(3 * s2 + 2) * NI + i2]};
+      double ea[5], eb[5], c2a, c2b, c3a, c3b;
+      proj_cell(l, i2 + 2, c2a, c2b);
+      proj_cell(l, i2 + 3, c3a, c3b);
+      proj_diff(l, i2, ea[0], eb[0]);
+      proj_diff(l, i2 + 1, ea[1], eb[1]);
+      proj_diff(l, i2 + 3, ea[3], eb[3]);
+      proj_diff(l, i2 + 4, ea[4], eb[4]);
+      ea[2] = c3a - c2a;
+      eb[2] = c3b - c2b;
+      const double al = (s2 == 0) ? alpha[0] : ((s2 == 1) ? alpha[1] : alpha[M - 1]);
       double d[5], q2;
-      if constexpr (SPLIT == 2) {
-        // The - side reconstructs its stencil negated: the reconstruction is odd in its data bit
-        // for bit (squares and comparisons do not see the sign; every other step is a rounded
-        // linear operation, and round-to-nearest is symmetric), so -weno(-d, -q2) is the value
-        // of MATH::side_diffs' stencil.  Its differences are then alpha-combined like the + side's,
-        // with -alpha, from the side-ordered products, and no selects are needed.
-        const unsigned long long sg = side2 ? 0x8000000000000000ull : 0ull;
-        const double sa = flip_sign(al, sg);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) d[k] = fma(sa, db[k], da[k]);
-        q2 = fma(al, b2, flip_sign(a2, sg));  // + side: a2 + alpha b2; - side: alpha b3 - a3
-        reconstruct_d(d, q2, side2 * (M * NI) + s * NI + i, sg);
-      } else {
-        MATH::side_diffs(da, db, a2, b2, a3, b3, al, false, d, q2);
-        reconstruct_d(d, q2, s * NI + i);
-        MATH::side_diffs(da, db, a2, b2, a3, b3, al, true, d, q2);
-        reconstruct_d(d, q2, M * NI + s * NI + i);
-      }
+      MATH::side_diffs(ea, eb, c2a, c2b, c3a, c3b, al, false, d, q2);
+      reconstruct_d(d, q2, s2 * NI + i2);
+      MATH::side_diffs(ea, eb, c2a, c2b, c3a, c3b, al, true, d, q2);
+      reconstruct_d(d, q2, M * NI + s2 * NI + i2);
     }
   } else if constexpr (IPT > 1) {
     // several items per thread: projection and both reconstructions of each item in turn, with
@@ -840,7 +1323,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   }
 
   // ---- D: interface fluxes h_{j+1/2} = R (F+ + F-)
-  const double* hsrc = s_F;
+  hsrc = s_F;
   if (FLUX == WT_FLUX_EULER1D) {
     for (int i = tid; i < ni; i += NT) {
       double rs[3] = {s_rs[i], s_rs[NI + i], s_rs[2 * NI + i]};
@@ -864,6 +1347,8 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
     }
     *phase ^= 1u;
   }
+  }
+
   // ---- E: flux difference, RK combine, ghost images, wave speeds.  Step-blocked: one
   // (cell, component) per thread, and no wave speeds (phase B of the next stage takes them).
   if (MODE == kStepBlocked && STAGE != STAGE_RHS) {
@@ -914,13 +1399,19 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   // where the screen does not apply); the FP64 speeds are then taken only for the cells that
   // can hold a maximum of the tile (below)
   constexpr bool kScreen = FLUX == WT_FLUX_EULER1D && MODE == kStage && STAGE != STAGE_RHS;
-  float* s_lam = reinterpret_cast<float*>(s_F);
+  float* s_lam = reinterpret_cast<float*>(CENTRAL ? s_L : s_F);
   float m32[3] = {0.0f, 0.0f, 0.0f};
   const float g32 = f32_hi(a.gamma * (a.gamma - 1.0));
   for (int t = tid; t < Tc; t += NT) {
     const long long j = js + t;
     const bool own = (MODE != kStepBlocked) || (j >= own_lo && j < own_hi);
     double uo[M];
+    // central stage tiles keep no window of u^n: one coalesced load per cell and component
+    double ug[M];
+    if constexpr (CENTRAL && MODE == kStage && kNeedUn) {
+#pragma unroll
+      for (int c = 0; c < M; ++c) ug[c] = a.un[c * a.pitch + j + G];
+    }
 #pragma unroll
     for (int c = 0; c < M; ++c) {
       // scalar fluxes: h = F+ + F- directly from the reconstruction
@@ -931,7 +1422,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         a.Lout[c * a.lout_stride + j] = L;
       } else {
         const double us = s_uin[c * W + off + t + G];
-        const double un = kNeedUn ? s_un[c * W + off + t + G] : us;
+        const double un = !kNeedUn ? us : ((CENTRAL && MODE == kStage) ? ug[c] : s_un[c * W + off + t + G]);
         uo[c] = MATH::template rk<(STAGE == STAGE_RHS ? 0 : STAGE)>(un, us, dt, L);
       }
     }
@@ -1048,11 +1539,11 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   return true;
 }
 
-template <class MATH, int FLUX, int STAGE, int T, int IPT = 1, bool REC = false>
+template <class MATH, int FLUX, int STAGE, int T, int IPT = 1, int USE = kForward>
 __device__ __forceinline__ bool stage1d_tile(const Stage1DArgs& a, const long long j0, const bool first_tile, double* sm,
                                              uint32_t& phase) {
   constexpr int M = FluxM<FLUX>::m;
-  using TL = TileOf<MATH, FLUX, T, 1, IPT, true>;
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT, USE>;
   constexpr int W = TL::W;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + TL::kBar);
   double* s_uin = sm + TL::kUin;
@@ -1115,7 +1606,7 @@ __device__ __forceinline__ bool stage1d_tile(const Stage1DArgs& a, const long lo
     ctl->active = 1;
   }
 
-  if (!stage1d_compute<MATH, FLUX, STAGE, T, kStage, IPT, REC>(a, j0, Tc, off, j0, j0 + Tc, alpha, dt, sm,
+  if (!stage1d_compute<MATH, FLUX, STAGE, T, kStage, IPT, USE>(a, j0, Tc, off, j0, j0 + Tc, alpha, dt, sm,
                                                               AlphaWait{0ull, 0, -1, 0, 0.0, 0.0, 0.0, 0.0}, &phase))
     return false;
   if (STAGE != STAGE_RHS) {
@@ -1127,23 +1618,23 @@ __device__ __forceinline__ bool stage1d_tile(const Stage1DArgs& a, const long lo
   return true;
 }
 
-template <class MATH, int FLUX, int STAGE, int T>
-__global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, 1, true>::NT) stage1d_kernel(const Stage1DArgs a) {
-  using TL = TileOf<MATH, FLUX, T, 1, 1, true>;
+template <class MATH, int FLUX, int STAGE, int T, int IPT>
+__global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) stage1d_kernel(const Stage1DArgs a) {
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT>;
   extern __shared__ __align__(16) double sm[];
   pdl_launch_dependents();
   if (threadIdx.x == 0) mbar_init(reinterpret_cast<uint64_t*>(sm + TL::kBar), 1);
   __syncthreads();
   pdl_wait();
   uint32_t phase = 0;
-  stage1d_tile<MATH, FLUX, STAGE, T>(a, (long long)blockIdx.x * T, blockIdx.x == 0, sm, phase);
+  stage1d_tile<MATH, FLUX, STAGE, T, IPT>(a, (long long)blockIdx.x * T, blockIdx.x == 0, sm, phase);
 }
 
 // Batched stage: a persistent grid walks a table of (problem, tile) work items over many
 // independent problems, each with its own grid, boundary conditions, alphas and dt.
-template <class MATH, int FLUX, int STAGE, int T, int IPT, bool REC = false>
+template <class MATH, int FLUX, int STAGE, int T, int IPT, int USE = kForward>
 __global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) stage1d_batched_kernel(const BatchArgs b) {
-  using TL = TileOf<MATH, FLUX, T, 1, IPT, true>;
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT, USE>;
   extern __shared__ __align__(16) double sm[];
   pdl_launch_dependents();
   if (threadIdx.x == 0) mbar_init(reinterpret_cast<uint64_t*>(sm + TL::kBar), 1);
@@ -1170,9 +1661,9 @@ __global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) s
     a.bc_lo = sg.bc_lo;
     a.bc_hi = sg.bc_hi;
     a.ctl = b.ctl + item.x;
-    a.rec = REC ? b.rec + (size_t)b.rec_off[item.x] * kAdjRec : nullptr;
+    a.rec = USE == kAdjRecord ? b.rec + (size_t)b.rec_off[item.x] * kAdjRec : nullptr;
     const long long j0 = (long long)item.y * T;
-    if (!stage1d_tile<MATH, FLUX, STAGE, T, IPT, REC>(a, j0, j0 == 0, sm, phase)) return;
+    if (!stage1d_tile<MATH, FLUX, STAGE, T, IPT, USE>(a, j0, j0 == 0, sm, phase)) return;
     __syncthreads();
   }
 }
@@ -1205,7 +1696,7 @@ __device__ __forceinline__ void load_halos(const double* uin, long long pitch, l
 template <class MATH, int FLUX, int T>
 __global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m>::NT, 3) persist1d_kernel(const PersistArgs p) {
   constexpr int M = FluxM<FLUX>::m;
-  using TL = TileOf<MATH, FLUX, T>;
+  using TL = KernelTile<MATH, FLUX, T, kResident>;
   constexpr int W = TL::W, NT = TL::NT;
   extern __shared__ __align__(16) double sm[];
   double* s_uin = sm + TL::kUin;
@@ -1386,11 +1877,11 @@ __device__ __forceinline__ bool sb_mailbox_halo(const unsigned long long* hi, co
 
 // one CTA per SM (the launch checks that the grid is co-resident)
 template <class MATH, int FLUX, int T>
-__global__ void __launch_bounds__(Tile1D<T + 4 * G, FluxM<FLUX>::m, 2>::NT, 1) stepblock1d_kernel(const PersistArgs p) {
+__global__ void __launch_bounds__(KernelTile<MATH, FLUX, T + 4 * G, kStepBlocked>::NT, 1) stepblock1d_kernel(const PersistArgs p) {
   constexpr int M = FluxM<FLUX>::m;
   constexpr int E0 = 3 * G;   // halo cells per side at the start of a step
   constexpr int TB = T + 4 * G;  // cells computed in stage 1: T + 2 * (E0 - G)
-  using TL = TileOf<MATH, FLUX, TB, 2>;
+  using TL = KernelTile<MATH, FLUX, TB, kStepBlocked>;
   constexpr int W = TL::W;
   static_assert(W >= T + 2 * E0, "window of a step");
   extern __shared__ __align__(16) double sm[];
@@ -1503,9 +1994,11 @@ cudaError_t launch_pdl(K kern, dim3 grid, dim3 block, size_t smem, cudaStream_t 
 }
 template <class MATH, int FLUX, int STAGE, int T>
 cudaError_t launch_stage1d_t(const Stage1DArgs& a, cudaStream_t st) {
-  using TL = TileOf<MATH, FLUX, T, 1, 1, true>;
+  // the central tiles' throughput form: one thread per interface
+  constexpr int IPT = (kCentralTile<MATH, FLUX, kForward> && T == 127) ? 3 : 1;
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT>;
   static_assert(TL::bytes <= 48 * 1024, "tile exceeds the default dynamic shared memory limit");
-  auto kern = stage1d_kernel<MATH, FLUX, STAGE, T>;
+  auto kern = stage1d_kernel<MATH, FLUX, STAGE, T, IPT>;
   const unsigned grid = (unsigned)((a.n + T - 1) / T);
   return launch_pdl(kern, dim3(grid), dim3(TL::NT), TL::bytes, st, a);
 }
@@ -1513,7 +2006,7 @@ cudaError_t launch_stage1d_t(const Stage1DArgs& a, cudaStream_t st) {
 // Cooperative launch of the persistent kernel (grid = number of tiles, all co-resident)
 template <class MATH, int FLUX, int T>
 cudaError_t launch_persist1d_t(const PersistArgs& p, int grid, cudaStream_t st) {
-  using TL = TileOf<MATH, FLUX, T>;
+  using TL = KernelTile<MATH, FLUX, T, kResident>;
   static_assert(TL::bytes <= 48 * 1024, "tile exceeds the default dynamic shared memory limit");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -1531,7 +2024,7 @@ cudaError_t launch_persist1d_t(const PersistArgs& p, int grid, cudaStream_t st) 
 // CTAs of the persistent kernel that fit on the device at once (0: no cooperative launch)
 template <class MATH, int FLUX, int T>
 int persist1d_capacity_t() {
-  using TL = TileOf<MATH, FLUX, T>;
+  using TL = KernelTile<MATH, FLUX, T, kResident>;
   int dev = 0, sms = 0, coop = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
@@ -1545,7 +2038,7 @@ int persist1d_capacity_t() {
 // Cooperative launch of the step-blocked kernel (grid = number of tiles of T cells)
 template <class MATH, int FLUX, int T>
 cudaError_t launch_stepblock1d_t(const PersistArgs& p, int grid, cudaStream_t st) {
-  using TL = TileOf<MATH, FLUX, T + 4 * G, 2>;
+  using TL = KernelTile<MATH, FLUX, T + 4 * G, kStepBlocked>;
   static_assert(TL::bytes <= 48 * 1024, "tile exceeds the default dynamic shared memory limit");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -1562,7 +2055,7 @@ cudaError_t launch_stepblock1d_t(const PersistArgs& p, int grid, cudaStream_t st
 
 template <class MATH, int FLUX, int T>
 int stepblock1d_capacity_t() {
-  using TL = TileOf<MATH, FLUX, T + 4 * G, 2>;
+  using TL = KernelTile<MATH, FLUX, T + 4 * G, kStepBlocked>;
   int dev = 0, sms = 0, coop = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
@@ -1573,24 +2066,29 @@ int stepblock1d_capacity_t() {
   return per * sms;
 }
 
+// tile: stepblock1d_tile
 template <class MATH>
-int stepblock1d_capacity_policy(int flux) {
-  switch (flux) {
-    case WT_FLUX_EULER1D: return stepblock1d_capacity_t<MATH, WT_FLUX_EULER1D, 27>();
-    case WT_FLUX_ADVECTION: return stepblock1d_capacity_t<MATH, WT_FLUX_ADVECTION, 51>();
-    case WT_FLUX_BURGERS: return stepblock1d_capacity_t<MATH, WT_FLUX_BURGERS, 51>();
+int stepblock1d_capacity_policy(int flux, int tile) {
+  if (flux == WT_FLUX_EULER1D) {
+    if (tile == 9) return stepblock1d_capacity_t<MATH, WT_FLUX_EULER1D, 9>();
+    if (tile == 18) return stepblock1d_capacity_t<MATH, WT_FLUX_EULER1D, 18>();
+    return tile == 27 ? stepblock1d_capacity_t<MATH, WT_FLUX_EULER1D, 27>() : 0;
   }
-  return 0;
+  if (tile != 51) return 0;
+  if (flux == WT_FLUX_ADVECTION) return stepblock1d_capacity_t<MATH, WT_FLUX_ADVECTION, 51>();
+  return flux == WT_FLUX_BURGERS ? stepblock1d_capacity_t<MATH, WT_FLUX_BURGERS, 51>() : 0;
 }
 
 template <class MATH>
-cudaError_t launch_stepblock1d_policy(int flux, const PersistArgs& p, int grid, cudaStream_t st) {
-  switch (flux) {
-    case WT_FLUX_EULER1D: return launch_stepblock1d_t<MATH, WT_FLUX_EULER1D, 27>(p, grid, st);
-    case WT_FLUX_ADVECTION: return launch_stepblock1d_t<MATH, WT_FLUX_ADVECTION, 51>(p, grid, st);
-    case WT_FLUX_BURGERS: return launch_stepblock1d_t<MATH, WT_FLUX_BURGERS, 51>(p, grid, st);
+cudaError_t launch_stepblock1d_policy(int flux, int tile, const PersistArgs& p, int grid, cudaStream_t st) {
+  if (flux == WT_FLUX_EULER1D) {
+    if (tile == 9) return launch_stepblock1d_t<MATH, WT_FLUX_EULER1D, 9>(p, grid, st);
+    if (tile == 18) return launch_stepblock1d_t<MATH, WT_FLUX_EULER1D, 18>(p, grid, st);
+    return tile == 27 ? launch_stepblock1d_t<MATH, WT_FLUX_EULER1D, 27>(p, grid, st) : cudaErrorInvalidValue;
   }
-  return cudaErrorInvalidValue;
+  if (tile != 51) return cudaErrorInvalidValue;
+  if (flux == WT_FLUX_ADVECTION) return launch_stepblock1d_t<MATH, WT_FLUX_ADVECTION, 51>(p, grid, st);
+  return flux == WT_FLUX_BURGERS ? launch_stepblock1d_t<MATH, WT_FLUX_BURGERS, 51>(p, grid, st) : cudaErrorInvalidValue;
 }
 
 // tiles with a persistent kernel: 31 and 63 (Euler), 63 (scalar fluxes); 0 for the others
@@ -1664,11 +2162,11 @@ cudaError_t launch_alpha1d_policy(int flux, const double* u, long long n, long l
   return cudaGetLastError();
 }
 
-template <class MATH, int FLUX, int STAGE, int T, int IPT, bool REC = false>
+template <class MATH, int FLUX, int STAGE, int T, int IPT, int USE = kForward>
 cudaError_t launch_stage1d_batched_t(const BatchArgs& b, int grid, cudaStream_t st) {
-  using TL = TileOf<MATH, FLUX, T, 1, IPT, true>;
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT, USE>;
   static_assert(TL::bytes <= 48 * 1024, "tile exceeds the default dynamic shared memory limit");
-  return launch_pdl(stage1d_batched_kernel<MATH, FLUX, STAGE, T, IPT, REC>, dim3(grid), dim3(TL::NT), TL::bytes, st,
+  return launch_pdl(stage1d_batched_kernel<MATH, FLUX, STAGE, T, IPT, USE>, dim3(grid), dim3(TL::NT), TL::bytes, st,
                     b);
 }
 
@@ -1676,19 +2174,19 @@ cudaError_t launch_stage1d_batched_t(const BatchArgs& b, int grid, cudaStream_t 
 template <class MATH>
 cudaError_t launch_stage1d_batched_record_policy(int stage, const BatchArgs& b, int grid, cudaStream_t st) {
   switch (stage) {
-    case STAGE_RK1: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK1, 127, 6, true>(b, grid, st);
-    case STAGE_RK2: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK2, 127, 6, true>(b, grid, st);
-    case STAGE_RK3: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK3, 127, 6, true>(b, grid, st);
+    case STAGE_RK1: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK1, 127, 6, kAdjRecord>(b, grid, st);
+    case STAGE_RK2: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK2, 127, 6, kAdjRecord>(b, grid, st);
+    case STAGE_RK3: return launch_stage1d_batched_t<MATH, WT_FLUX_EULER1D, STAGE_RK3, 127, 6, kAdjRecord>(b, grid, st);
   }
   return cudaErrorInvalidValue;
 }
 
-template <class MATH, int FLUX, int T, int IPT = 1>
+template <class MATH, int FLUX, int T, int IPT = 1, int USE = kForward>
 cudaError_t launch_stage1d_batched_flux(int stage, const BatchArgs& b, int grid, cudaStream_t st) {
   switch (stage) {
-    case STAGE_RK1: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK1, T, IPT>(b, grid, st);
-    case STAGE_RK2: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK2, T, IPT>(b, grid, st);
-    case STAGE_RK3: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK3, T, IPT>(b, grid, st);
+    case STAGE_RK1: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK1, T, IPT, USE>(b, grid, st);
+    case STAGE_RK2: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK2, T, IPT, USE>(b, grid, st);
+    case STAGE_RK3: return launch_stage1d_batched_t<MATH, FLUX, STAGE_RK3, T, IPT, USE>(b, grid, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -1706,6 +2204,9 @@ cudaError_t launch_stage1d_batched_policy(int flux, int stage, int tile, const B
     if (tile == 2127) return launch_stage1d_batched_flux<MATH, WT_FLUX_EULER1D, 127, 3>(stage, b, grid, st);
     if (tile == 3127) return launch_stage1d_batched_flux<MATH, WT_FLUX_EULER1D, 127, 4>(stage, b, grid, st);
     if (tile == 5127) return launch_stage1d_batched_flux<MATH, WT_FLUX_EULER1D, 127, 6>(stage, b, grid, st);
+    if (tile == kTileAdjForward)
+      return launch_stage1d_batched_flux<MATH, WT_FLUX_EULER1D, 127, 6, MATH::kCentral ? kAdjForward : kForward>(
+          stage, b, grid, st);
   } else if (flux == WT_FLUX_ADVECTION) {
     if (tile == 63) return launch_stage1d_batched_flux<MATH, WT_FLUX_ADVECTION, 63>(stage, b, grid, st);
     if (tile == 127) return launch_stage1d_batched_flux<MATH, WT_FLUX_ADVECTION, 127>(stage, b, grid, st);
@@ -1716,11 +2217,11 @@ cudaError_t launch_stage1d_batched_policy(int flux, int stage, int tile, const B
   return cudaErrorInvalidValue;
 }
 
-template <class MATH, int FLUX, int T, int IPT = 1>
+template <class MATH, int FLUX, int T, int IPT = 1, int USE = kForward>
 int batched_occupancy_t() {
-  using TL = TileOf<MATH, FLUX, T, 1, IPT, true>;
+  using TL = KernelTile<MATH, FLUX, T, kStage, IPT, USE>;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stage1d_batched_kernel<MATH, FLUX, STAGE_RK2, T, IPT>,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stage1d_batched_kernel<MATH, FLUX, STAGE_RK2, T, IPT, USE>,
                                                     TL::NT, TL::bytes) != cudaSuccess)
     return 0;
   return nb;
@@ -1737,6 +2238,8 @@ int batched_occupancy_policy(int flux, int tile) {
     if (tile == 2127) return batched_occupancy_t<MATH, WT_FLUX_EULER1D, 127, 3>();
     if (tile == 3127) return batched_occupancy_t<MATH, WT_FLUX_EULER1D, 127, 4>();
     if (tile == 5127) return batched_occupancy_t<MATH, WT_FLUX_EULER1D, 127, 6>();
+    if (tile == kTileAdjForward)
+      return batched_occupancy_t<MATH, WT_FLUX_EULER1D, 127, 6, MATH::kCentral ? kAdjForward : kForward>();
   } else if (flux == WT_FLUX_ADVECTION) {
     if (tile == 63) return batched_occupancy_t<MATH, WT_FLUX_ADVECTION, 63>();
     if (tile == 127) return batched_occupancy_t<MATH, WT_FLUX_ADVECTION, 127>();

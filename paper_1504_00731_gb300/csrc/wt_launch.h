@@ -74,6 +74,8 @@ struct BatchArgs {
 // tile: a tile code, cells per tile + 1000 x (items per thread - 1): 31, 63, 127 (Euler; 63, 127
 // scalar) with one (interface, field) item per thread, 1063 and 1127 (Euler) with two,
 // 2127, 3127 and 5127 (Euler) with three, four and six
+// kTileAdjForward (Euler): 5127 with every reconstruction projected, for the adjoint's forward pass
+constexpr int kTileAdjForward = -5127;
 cudaError_t launch_stage1d_batched_strict(int flux, int stage, int tile, const BatchArgs& b, int grid, cudaStream_t st);
 cudaError_t launch_stage1d_batched_fast(int flux, int stage, int tile, const BatchArgs& b, int grid, cudaStream_t st);
 // the adjoint's recording forward stage (1D Euler, tile code 5127): also writes b.rec
@@ -193,13 +195,18 @@ Stage1DArgs base_args(const wt_problem* p, long long n, double dx, long long pit
 cudaError_t launch_persist1d_strict(int flux, int tile, const PersistArgs& p, int grid, cudaStream_t st);
 cudaError_t launch_persist1d_fast(int flux, int tile, const PersistArgs& p, int grid, cudaStream_t st);
 int persist1d_capacity_strict(int flux, int tile);
-// tile of the step-blocked kernel: 27 cells (Euler: 3 x 40 interface items = 4 warps in stage
-// 1), 51 cells (scalar fluxes: 64 items = 2 warps)
-inline int stepblock1d_tile(int flux) { return flux == WT_FLUX_EULER1D ? 27 : 51; }
-cudaError_t launch_stepblock1d_strict(int flux, const PersistArgs& p, int grid, cudaStream_t st);
-cudaError_t launch_stepblock1d_fast(int flux, const PersistArgs& p, int grid, cudaStream_t st);
-int stepblock1d_capacity_strict(int flux);
-int stepblock1d_capacity_fast(int flux);
+// tile of the step-blocked kernel: the smallest that needs at most one CTA per SM, 9, 18 or 27 cells
+// (Euler), 51 cells (scalar fluxes).  A stage lasts as long as the FP64 work of the tile holding a
+// shock: with 9 cells (22 interfaces in stage 1, 5 warps) instead of 27 (40 interfaces, 8 warps
+// on 4 FP64 pipes) a 300-cell run to t = 1.3 takes 11.2 ms instead of 14.3.
+inline int stepblock1d_tile(int flux, long long n, int sms) {
+  if (flux != WT_FLUX_EULER1D) return 51;
+  return n <= 9LL * sms ? 9 : (n <= 18LL * sms ? 18 : 27);
+}
+cudaError_t launch_stepblock1d_strict(int flux, int tile, const PersistArgs& p, int grid, cudaStream_t st);
+cudaError_t launch_stepblock1d_fast(int flux, int tile, const PersistArgs& p, int grid, cudaStream_t st);
+int stepblock1d_capacity_strict(int flux, int tile);
+int stepblock1d_capacity_fast(int flux, int tile);
 int persist1d_capacity_fast(int flux, int tile);
 cudaError_t launch_stage1d_strict(int flux, int stage, int tile, const Stage1DArgs& a, cudaStream_t st);
 cudaError_t launch_stage1d_fast(int flux, int stage, int tile, const Stage1DArgs& a, cudaStream_t st);

@@ -55,6 +55,20 @@ struct FastMath {
     double ir;
     euler_cell_ir(U, gamma, f, u, H, sr, p, ir);
   }
+  // the central tiles' cell quantities (wt_central.cuh): f, u and H; sqrt(rho) is taken only where an
+  // interface needs Roe's average in FP64
+  static constexpr bool kCentral = true;
+  __device__ __forceinline__ static void euler_cell_flux(const double* U, double gamma, double* f, double& u, double& H) {
+    const double ir = 1.0 / U[0];
+    u = __dmul_rn(U[1], ir);
+    const double p = __dmul_rn(gamma - 1.0, fma(-0.5 * U[1], u, U[2]));
+    const double e = __dadd_rn(U[2], p);
+    f[0] = U[1];
+    f[1] = fma(U[1], u, p);
+    f[2] = __dmul_rn(e, u);
+    H = __dmul_rn(e, ir);
+  }
+  __device__ __forceinline__ static double sqrt_rho(double rho) { return __dmul_rn(rho, rsqrt(rho)); }
   // sound speed c = sqrt(c2) as c2 rsqrt(c2), a shorter dependent chain than the IEEE square
   // root (the wave speeds open the alpha exchange of every stage); c2 <= 0, huge or NaN keeps
   // the square root
@@ -372,32 +386,32 @@ struct FastMath {
   __device__ __forceinline__ static bool weno_front(const double* q, double eps, double alpha_R, double& out,
                                                     double* rec) {
     const double d0 = q[1] - q[0], d1 = q[2] - q[1], d2 = q[3] - q[2], d3 = q[4] - q[3], d4 = q[5] - q[4];
-    return weno_front_core<false>(d0, d1, d2, d3, d4, q[2], q[3], eps, alpha_R, out, rec);
+    const int scr = weno_front_core<false>(d0, d1, d2, d3, d4, q[2], q[3], eps, alpha_R, rec);
+    if (scr != 0) out = linear_theta(d0, d1, d2, d3, d4, q[2], scr == 1);
+    return scr != 0;
   }
-  // the same from the stencil's differences and q_2 (q_3 taken as q_2 + d_2)
-  __device__ __forceinline__ static bool weno_front_d(const double* d, double q2, double eps, double alpha_R,
-                                                      double& out, double* rec) {
-    return weno_front_core<true>(d[0], d[1], d[2], d[3], d[4], q2, 0.0, eps, alpha_R, out, rec);
+  // the same from the stencil's differences and q_2 (q_3 taken as q_2 + d_2), the linear scheme left
+  // to the caller: returns the screen's verdict, 1 (theta = 1), 2 (theta = 0) or 0 (a record)
+  __device__ __forceinline__ static int weno_front_d(const double* d, double q2, double eps, double alpha_R,
+                                                     double* rec) {
+    return weno_front_core<true>(d[0], d[1], d[2], d[3], d[4], q2, 0.0, eps, alpha_R, rec);
   }
   template <bool Q3D>
-  __device__ __forceinline__ static bool weno_front_core(double d0, double d1, double d2, double d3, double d4,
-                                                         double q2, double q3, double eps, double alpha_R,
-                                                         double& out, double* rec) {
+  __device__ __forceinline__ static int weno_front_core(double d0, double d1, double d2, double d3, double d4,
+                                                        double q2, double q3, double eps, double alpha_R,
+                                                        double* rec) {
     const double s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
     const double t5b = s2 - s1;
     const double t5a = fma(-2.0, s1, s0) + s2;
     const double t6a = fma(-3.0, t5b, s3 - s0);
     const double t6b = (s0 + s3) - (s1 + s2);
     const int scr = screen(s0, s1, s2, s3, d1, d2, d3, t5a, t5b, t6a, t6b, eps, alpha_R);
-    if (scr != 0) {
-      out = linear_theta(d0, d1, d2, d3, d4, q2, scr == 1);
-      return true;
-    }
+    if (scr != 0) return scr;
     rec[0] = d0; rec[1] = d1; rec[2] = d2; rec[3] = d3; rec[4] = d4;
     rec[5] = s0; rec[6] = s1; rec[7] = s2; rec[8] = s3;
     rec[9] = t5a; rec[10] = t5b; rec[11] = t6a; rec[12] = t6b;
     rec[13] = q2; rec[14] = Q3D ? q2 + d2 : q3;
-    return false;
+    return 0;
   }
 
   // Lane k (0..3) of the quad of lanes `qmask` completes a deferred stencil: indicator k
@@ -419,17 +433,15 @@ struct FastMath {
     const double bk = fma((k == 3 ? C1348 : C1312) * x, x, y * y);
     const double x1 = __shfl_xor_sync(qmask, bk, 1), x2 = __shfl_xor_sync(qmask, bk, 2),
                  x3 = __shfl_xor_sync(qmask, bk, 3);
-    // indicator j comes from the lane at xor distance j ^ k
-    const double b0 = k == 0 ? bk : (k == 1 ? x1 : (k == 2 ? x2 : x3));
-    const double b1 = k == 1 ? bk : (k == 0 ? x1 : (k == 3 ? x2 : x3));
-    const double b2 = k == 2 ? bk : (k == 3 ? x1 : (k == 0 ? x2 : x3));
-    const double b3 = k == 3 ? bk : (k == 2 ? x1 : (k == 1 ? x2 : x3));
-    const double tau5 = fma(C1312 * t5a, t5a, t5b * t5b);
-    const double tau6 = fma(C1312 * t6a, t6a, 0.25 * (t6b * t6b));
+    // tau5 on the even lanes, tau6 on the odd ones (0.25 (y y) = (0.5 y)^2 exactly)
+    const bool odd = k & 1;
+    const double tx = odd ? t6a : t5a, ty = odd ? 0.5 * t6b : t5b;
+    const double tk = fma(C1312 * tx, tx, ty * ty), to = __shfl_xor_sync(qmask, tk, 1);
+    const double tau5 = odd ? to : tk, tau6 = odd ? tk : to;
     const bool theta1 = !(bits(tau6) < bits(tau5));
     const double tau = theta1 ? tau5 : tau6;
-    const double bmax = nmax(nmax(b0, b1), nmax(b2, b3));
-    const double bmin = nmin(nmin(b0, b1), nmin(b2, b3));
+    const double bmax = nmax(nmax(bk, x1), nmax(x2, x3));
+    const double bmin = nmin(nmin(bk, x1), nmin(x2, x3));
     if (!(bits(fma(alpha_R, bmin, alpha_R * eps)) < bits(bmax))) return linear_theta(d0, d1, d2, d3, d4, q2, theta1);
     // Eqs. (fh0)-(fh3): fh_k = fma(A, X, fma(B, Y, Z))
     const double A = k == 0 ? 5.0 / 6.0 : (k == 1 ? 1.0 / 6.0 : (k == 2 ? 2.0 / 3.0 : 1.0 / 3.0));
@@ -438,7 +450,14 @@ struct FastMath {
     const double Y = k == 0 ? d0 : (k == 1 ? d2 : d3);
     const double Z = k == 3 ? q3 : q2;
     const double fhk = fma(A, X, fma(B, Y, Z));
-    const double e[4] = {eps + b0, eps + b1, eps + b2, eps + b3};
+    // eps + beta_k, taken on its lane; term j comes from the lane at xor distance j ^ k
+    const double ek = eps + bk;
+    const double y1 = __shfl_xor_sync(qmask, ek, 1), y2 = __shfl_xor_sync(qmask, ek, 2),
+                 y3 = __shfl_xor_sync(qmask, ek, 3);
+    const double e[4] = {k == 0 ? ek : (k == 1 ? y1 : (k == 2 ? y2 : y3)),
+                         k == 1 ? ek : (k == 0 ? y1 : (k == 3 ? y2 : y3)),
+                         k == 2 ? ek : (k == 3 ? y1 : (k == 0 ? y2 : y3)),
+                         k == 3 ? ek : (k == 2 ? y1 : (k == 1 ? y2 : y3))};
     double wk, nk;
     weno_weight(k, e, tau, theta1, fhk, wk, nk);
     wk += __shfl_xor_sync(qmask, wk, 1);
@@ -504,6 +523,16 @@ struct FastMath {
     h[0] = s02 + F[1];
     h[1] = fma(u, h[0], c * d20);
     h[2] = fma(H, s02, fma(u * c, d20, 0.5 * u * u * F[1]));
+  }
+
+  // component c of it, the same value
+  __device__ __forceinline__ static double backproject_c(int c, const double* rs, const double* F) {
+    const double u = rs[0], H = rs[1], cc = rs[2];
+    const double s02 = F[0] + F[2];
+    if (c == 0) return s02 + F[1];
+    const double d20 = F[2] - F[0];
+    if (c == 1) return fma(u, s02 + F[1], cc * d20);
+    return fma(H, s02, fma(u * cc, d20, 0.5 * u * u * F[1]));
   }
 
   // rounded on its own (never contracted into the sum of the two sweeps), so that

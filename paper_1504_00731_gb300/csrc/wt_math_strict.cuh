@@ -10,6 +10,7 @@ namespace wt {
 
 struct StrictMath {
   static constexpr bool kStrict = true;
+  static constexpr bool kCentral = false;  // no central screen (wt_central.cuh): every reconstruction is evaluated
   static constexpr bool kRoeRows = false;  // the whole Roe matrix per interface (roe)
   // projection v = kProj (L f +- alpha L u) with the stored L = kLScale * L_true
   static constexpr double kProj = 0.5, kLScale = 1.0;
