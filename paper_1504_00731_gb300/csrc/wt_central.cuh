@@ -247,6 +247,95 @@ __device__ __forceinline__ bool prove_field(const float* a, const float* b, cons
   return ok;
 }
 
+// ---- 2D (Sec. 4.3): normal velocity u and tangential velocity t of a sweep.  Projections with w1 = xn - u
+// x0, wt = xt - t x0, w2 = xE - u (xn + w1) / 2 - t (xt + wt) / 2; the shear field is wt itself, the
+// others are those of 1D.
+struct Roe32Shear {
+  Roe32 r;
+  float t, T;
+};
+__device__ __forceinline__ Roe32Shear roe32_2d(double ra_, double na_, double ta_, double Ha_, double rb_, double nb_,
+                                               double tb_, double Hb_, float gm1) {
+  Roe32Shear o;
+  Roe32& r = o.r;
+  const float ra = f32_trunc(ra_), rb = f32_trunc(rb_), ua = f32_trunc(na_), ub = f32_trunc(nb_);
+  const float ta = f32_trunc(ta_), tb = f32_trunc(tb_), Ha = f32_trunc(Ha_), Hb = f32_trunc(Hb_);
+  const float sa = fmul(ra, frsqrt_hw(ra)), sb = fmul(rb, frsqrt_hw(rb));
+  const float hw = fmul(fmul(0.5f, fsub(sa, sb)), frcp_hw(fadd(sa, sb)));
+  const float du = fsub(ua, ub), dt = fsub(ta, tb);
+  r.u = ffma(hw, du, fmul(0.5f, fadd(ua, ub)));
+  o.t = ffma(hw, dt, fmul(0.5f, fadd(ta, tb)));
+  const float H = ffma(hw, fsub(Ha, Hb), fmul(0.5f, fadd(Ha, Hb)));
+  r.U = fmaxf(fabsf(ua), fabsf(ub));
+  o.T = fmaxf(fabsf(ta), fabsf(tb));
+  const float he = ffma(-0.5f, fadd(fmul(r.u, r.u), fmul(o.t, o.t)), H);
+  const float big = fadd(fadd(fmul(r.U, r.U), fmul(o.T, o.T)), fmaxf(fabsf(Ha), fabsf(Hb)));
+  const float c2 = fmul(gm1, he);
+  r.ic = frsqrt_hw(c2);
+  r.b1 = fmul(gm1, fmul(r.ic, r.ic));
+  r.rel = ffma(0x1p-19f, fmul(big, r.b1), 0x1p-20f);
+  // (one more product and sum than in 1D: 2.75 * 2^-23 beside E / U, still below 1.5 * 2^-21)
+  r.q = ffma(0x1p-20f, fmaxf(fmul(fabsf(du), frcp_hw(fadd(r.U, 1e-30f))), fmul(fabsf(dt), frcp_hw(fadd(o.T, 1e-30f)))),
+             0x1.8p-21f);
+  r.thr = fmul(fmul(60.0f * 0x1p-53f, fminf(ra, rb)), ffma(c2, r.ic, fabsf(r.u)));
+  r.ok = ra > 0x1p-60f && rb > 0x1p-60f && ra < 0x1p60f && rb < 0x1p60f && fmul(he, 32.0f) >= big && big < 0x1p60f &&
+         big > 0x1p-60f;
+  return o;
+}
+// fields 0..3 (u - c, u, shear, u + c) of one array (f or u), as take_field: a field's projections and errors
+struct Proj32Shear {
+  float2 jk[9];
+  float x0[9], wt[9];
+  float2 nb[5];
+  float nt[5];
+  float jm, km, xm, tm;
+};
+__device__ __forceinline__ void project_stencil_2d(const Roe32Shear& o, const float (*d)[5], const float4* h,
+                                                   Proj32Shear& p) {
+  const Roe32& r = o.r;
+  p.jm = p.km = p.xm = p.tm = 0.0f;
+  float mx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int v = 0; v < 9; ++v) {
+    float x[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) x[c] = v < 5 ? d[c][v < 5 ? v : 0] : (v == 5 ? h[c].x : (v == 6 ? h[c].y : (v == 7 ? h[c].z : h[c].w)));
+    const float w1 = ffma(-r.u, x[0], x[1]), wt = ffma(-o.t, x[0], x[2]);
+    const float w2 = ffma(fmul(-0.5f, o.t), fadd(x[2], wt), ffma(fmul(-0.5f, r.u), fadd(x[1], w1), x[3]));
+    p.jk[v] = make_float2(fmul(r.ic, w1), fmul(r.b1, w2));
+    p.x0[v] = x[0];
+    p.wt[v] = wt;
+    if (v < 5) {
+      p.jm = fmaxf(p.jm, fabsf(p.jk[v].x));
+      p.km = fmaxf(p.km, fabsf(p.jk[v].y));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) mx[c] = fmaxf(mx[c], fabsf(x[c]));
+    }
+    if (v >= 4) {  // the bounds of the largest cell difference, then of the high differences
+      const int b = v - 4;
+      if (b == 0) p.xm = mx[0];
+      const float y0 = b == 0 ? mx[0] : fabsf(x[0]), y1 = b == 0 ? mx[1] : fabsf(x[1]),
+                  y2 = b == 0 ? mx[2] : fabsf(x[2]), y3 = b == 0 ? mx[3] : fabsf(x[3]);
+      const float n1 = ffma(r.U, y0, y1), nt = ffma(o.T, y0, y2);
+      p.nb[b] = make_float2(fmul(r.ic, n1), fmul(r.b1, ffma(o.T, nt, ffma(r.U, n1, y3))));
+      p.nt[b] = nt;
+    }
+  }
+}
+__device__ __forceinline__ void take_field_2d(int s, const Roe32Shear& o, const Proj32Shear& p, float* a, float* ea) {
+  const Roe32& r = o.r;
+  const int s1 = s == 3 ? 2 : s;  // the 1D field's number (s != 2)
+#pragma unroll
+  for (int k = 0; k < 9; ++k) a[k] = s == 2 ? p.wt[k] : field32(s1, p.jk[k], p.x0[k]);
+  ea[0] = s == 2 ? fmul(r.q, p.nt[0]) : field_err(s1, r, p.nb[0], p.jm, p.km, p.xm);
+  const float pe = fmul(0x1p-40f, s == 2 ? p.nt[0] : (s == 1 ? fadd(p.xm, p.nb[0].y) : fadd(p.nb[0].x, p.nb[0].y)));
+#pragma unroll
+  for (int v = 0; v < 4; ++v)
+    ea[1 + v] = fadd(pe, s == 2 ? fmul(r.q, p.nt[1 + v])
+                                : field_err(s1, r, p.nb[1 + v], fabsf(p.jk[5 + v].x), fabsf(p.jk[5 + v].y),
+                                            fabsf(p.x0[5 + v])));
+}
+
 // the sixth-order central value (Eq. (fh_6)) from the two centre values and the outer four
 // differences d_0, d_1, d_3, d_4: (q2 + q3) / 2 + (7 (d1 - d3) - (d0 - d4)) / 60, the same value
 // for mirrored data

@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) alpha1d_kernel(const double* __restrict__
     } else {
       double x = u[j + G];
       double lam = (FLUX == WT_FLUX_ADVECTION) ? fabs(adv) : fabs(x);
-      if (!isfinite(x)) flag_error(ctl, WT_ERR_NONPHYSICAL);
+      if (!finite1(x)) flag_error(ctl, WT_ERR_NONPHYSICAL);
       key_max(v[0], lam);
     }
   }
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(256) alpha1d_batched_kernel(const double* __re
     } else {
       double x = up[j + G];
       double lam = (FLUX == WT_FLUX_ADVECTION) ? fabs(adv) : fabs(x);
-      if (!isfinite(x)) flag_error(c, WT_ERR_NONPHYSICAL);
+      if (!finite1(x)) flag_error(c, WT_ERR_NONPHYSICAL);
       key_max(v[0], lam);
     }
   }
@@ -934,7 +934,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         if constexpr (!CENTRAL) s_sr[k] = sr;
       } else {
         const double xv = U[0];
-        if (!isfinite(xv)) flag_error(ctl, WT_ERR_NONPHYSICAL);
+        if (!finite1(xv)) flag_error(ctl, WT_ERR_NONPHYSICAL);
         s_f[k] = (FLUX == WT_FLUX_ADVECTION) ? MATH::flux_advection(a.adv_speed, xv) : MATH::flux_burgers(xv);
       }
     }
@@ -1365,7 +1365,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
       if (STAGE == STAGE_RK3) {
         s_un[c * W + off + t + G] = v;
         if (j >= own_lo && j < own_hi) {
-          if (!isfinite(v)) flag_error(ctl, WT_ERR_NONPHYSICAL);
+          if (!finite1(v)) flag_error(ctl, WT_ERR_NONPHYSICAL);
           double* o = a.uout + c * a.pitch;
           o[j + G] = v;
           // the halo mailbox: u^{n+1} for the neighbours' next step, two tagged words
@@ -1454,7 +1454,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         }
       }
       if (own && MODE == kStepBlocked) {
-        if (FLUX == WT_FLUX_EULER1D ? !finite3(uo) : !isfinite(uo[0])) flag_error(ctl, WT_ERR_NONPHYSICAL);
+        if (FLUX == WT_FLUX_EULER1D ? !finite3(uo) : !finite1(uo[0])) flag_error(ctl, WT_ERR_NONPHYSICAL);
       } else if (own) {
         if constexpr (kScreen) {
           if (!finite3(uo)) flag_error(ctl, WT_ERR_NONPHYSICAL);
@@ -1476,7 +1476,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
           for (int f = 0; f < M; ++f) key_max(vmax[f], lam[f]);
         } else {
           const double lam = (FLUX == WT_FLUX_ADVECTION) ? fabs(a.adv_speed) : fabs(uo[0]);
-          if (!isfinite(uo[0])) flag_error(ctl, WT_ERR_NONPHYSICAL);
+          if (!finite1(uo[0])) flag_error(ctl, WT_ERR_NONPHYSICAL);
           key_max(vmax[0], lam);
         }
       }
@@ -1994,8 +1994,8 @@ cudaError_t launch_pdl(K kern, dim3 grid, dim3 block, size_t smem, cudaStream_t 
 }
 template <class MATH, int FLUX, int STAGE, int T>
 cudaError_t launch_stage1d_t(const Stage1DArgs& a, cudaStream_t st) {
-  // the central tiles' throughput form: one thread per interface
-  constexpr int IPT = (kCentralTile<MATH, FLUX, kForward> && T == 127) ? 3 : 1;
+  // the central tiles' throughput form
+  constexpr int IPT = (kCentralTile<MATH, FLUX, kForward> && T == 127) ? 6 : 1;
   using TL = KernelTile<MATH, FLUX, T, kStage, IPT>;
   static_assert(TL::bytes <= 48 * 1024, "tile exceeds the default dynamic shared memory limit");
   auto kern = stage1d_kernel<MATH, FLUX, STAGE, T, IPT>;

@@ -4,10 +4,13 @@
 //   alpha2d             alpha_s per direction and the 2D CFL quantity (warp-shuffle maxima)
 //   stage2d             fused RHS + RK stage: a TX x TY tile plus its 3-cell halo staged row by
 //                       row with bulk copies, the x sweep then the y sweep in shared memory,
-//                       one output write per cell; 104 KB of shared memory, so that two
-//                       CTAs (16 warps) share an SM
+//                       one output write per cell; at most 112 KB of shared memory per 256
+//                       threads, so that 16 warps share an SM
 #pragma once
 
+#include <type_traits>
+
+#include "wt_central.cuh"
 #include "wt_device.cuh"
 #include "wt_launch.h"
 
@@ -41,9 +44,208 @@ struct Tile2D {
   static constexpr int kTotal = kF + 4 * NI;
   static_assert(16 * NI >= 9 * 32, "reduction scratch inside the eigenvector buffer");
   static constexpr size_t bytes = sizeof(double) * kTotal;
+  static constexpr int kCtas = 2;
   // two CTAs per SM: 228 KB of shared memory per SM, 1 KB of it reserved per CTA
   static_assert(2 * (bytes + 1024) <= 228 * 1024, "two tiles must fit on one SM");
 };
+
+// What the fast policy's kernel costs: about 190 FP64 thread instructions per cell and stage where the data
+// are smooth (1245 with every interface projected), 58 % of the FP64 pipe's cycles at 16 warps per
+// SM; 2048 x 2048 vortices 59.8 -> 18.1 ms for two steps, 120 x 360 Rayleigh-Taylor 22.3 -> 13.6
+// ms for 40 (a fifth of its y interfaces are on fronts and take the FP64 path).
+//
+// Tile of the central screen (wt_central.cuh; the fast policy): no eigenvector or reconstruction
+// buffers per interface; the differences along the sweep as FP32 pairs, f's also in FP64 for
+// the central fluxes, in one buffer for both sweeps.
+template <int TX, int TY>
+struct Tile2DC {
+  static constexpr int WX = TX + 2 * G;
+  static constexpr int RY = TY + 2 * G;
+  static constexpr int NCELL = WX * RY;
+  static constexpr int NIX = (TX + 1) * TY;
+  static constexpr int NIY = TX * (TY + 1);
+  static constexpr int NI = NIX > NIY ? NIX : NIY;
+  static constexpr int NT = TX * 8;
+  static_assert(NIX <= NT && NIY <= NT, "one interface per thread");
+  static constexpr int kCtas = 512 / NT;  // per SM
+  static_assert(TX * TY <= NT, "one cell per thread in the flux difference and the stage update");
+  static constexpr int NDX = (TX + 5) * TY, NDY = TX * (TY + 5);  // differences of a sweep
+  static constexpr int ND = NDX > NDY ? NDX : NDY;
+  static constexpr int FC = 64;  // listed interfaces taken at a time
+  static constexpr int kBar = 0;
+  static constexpr int kUin = 2;
+  static constexpr int kU = kUin + 4 * NCELL;
+  static constexpr int kV = kU + NCELL;
+  static constexpr int kH = kV + NCELL;
+  static constexpr int kFg = kH + NCELL;               // [4][NCELL] f, then g
+  static constexpr int kDf = kFg + 4 * NCELL;          // [4][ND] differences of the sweep's flux
+  static constexpr int kPair = kDf + 4 * ND;           // [8][ND] differences of flux and state, FP32 pairs
+  static constexpr int kL = kPair;                     // FP64 path: [16][FC], then [4][FC], [4][FC]
+  static constexpr int kRs = kL + 16 * FC;
+  static constexpr int kF = kRs + 4 * FC;
+  static_assert(24 * FC <= 8 * ND, "the FP64 path's buffers over the pairs");
+  static constexpr int kHf = kPair + 8 * ND;           // [4][NI]
+  static constexpr int kRed = kHf + 4 * NI;            // maxima of the speeds
+  static constexpr int kList = kRed + 48;              // ints [NI], and a counter each for the list and the speeds
+  static constexpr int kTotal = kList + (NI + 1) / 2 + 2;
+  static constexpr size_t bytes = sizeof(double) * kTotal;
+  static_assert(kCtas * (bytes + 1024) <= 228 * 1024, "512 threads' tiles must fit on one SM");
+};
+// Rows per tile: with 7 every interface of a sweep has its own thread (231 and 256 of 256, 119 and 128 of
+// 128); with 8 a second pass over 8 and 32 of them costs as long as the first.
+template <class MATH>
+constexpr int kTileY = MATH::kCentral ? 7 : 8;
+template <class MATH, int TX, int TY>
+using KernelTile2D = std::conditional_t<MATH::kCentral, Tile2DC<TX, TY>, Tile2D<TX, TY>>;
+
+// One sweep's interface fluxes by the central screen (as central_fluxes in 1D): DIR 0 the x sweep
+// (interface i of row r at r (tcx + 1) + i), 1 the y sweep (interface j of column t at j tcx + t).
+template <class MATH, int DIR, class TL, int TX>
+__device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tcx, const int tcy,
+                                              const double (&alpha)[4], double* sm) {
+  constexpr int WX = TL::WX, NCELL = TL::NCELL, NI = TL::NI, NT = TL::NT, ND = TL::ND, FC = TL::FC;
+  constexpr int ST = DIR == 0 ? 1 : WX;   // cell stride along the sweep
+  constexpr int SD = DIR == 0 ? 1 : TX;   // stride of the differences along the sweep
+  constexpr int PD = DIR == 0 ? TX + 5 : TX;  // their row pitch
+  constexpr int N1 = 1 + DIR, T1 = 2 - DIR;   // components: normal and tangential momentum
+  const int tid = threadIdx.x;
+  double* s_uin = sm + TL::kUin;
+  double* s_n = sm + (DIR == 0 ? TL::kU : TL::kV);
+  double* s_t = sm + (DIR == 0 ? TL::kV : TL::kU);
+  double* s_H = sm + TL::kH;
+  double* s_fg = sm + TL::kFg;
+  double* s_df = sm + TL::kDf;
+  float2* s_pair = reinterpret_cast<float2*>(sm + TL::kPair);
+  double* s_h = sm + TL::kHf;
+  int* s_list = reinterpret_cast<int*>(sm + TL::kList);
+  int* s_nl = s_list + NI;
+  // components in the sweep's order (density, normal momentum, tangential momentum, energy)
+  auto comp = [](int c) { return c == 1 ? N1 : (c == 2 ? T1 : c); };
+  const int nper = DIR == 0 ? tcx + 1 : tcx;  // interfaces per row of the tile
+  const int ni = DIR == 0 ? (tcx + 1) * tcy : tcx * (tcy + 1);
+  // ---- D1
+  const int drow = DIR == 0 ? tcx + 5 : tcx, dn = DIR == 0 ? drow * tcy : drow * (tcy + 5);
+  for (int q = tid; q < dn; q += NT) {
+    const int r = q / drow, col = q - r * drow;
+    const int k = DIR == 0 ? (r + G) * WX + col : r * WX + col + G;
+    const int p = r * PD + col;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double* x = s_fg + comp(c) * NCELL + k;
+      const double df = __dsub_rn(x[ST], x[0]);
+      s_df[c * ND + p] = df;
+      s_pair[c * ND + p] = f32_pair(df);
+      const double* y = s_uin + comp(c) * NCELL + k;
+      s_pair[(4 + c) * ND + p] = f32_pair(__dsub_rn(y[ST], y[0]));
+    }
+  }
+  if (tid == 0) *s_nl = 0;
+  __syncthreads();
+  // ---- D2
+  const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
+  const bool screenable = fmul(aR, eps) > 1e-30f;
+  for (int it = tid; it < ni; it += NT) {
+    const int r = it / nper, i = it - r * nper;
+    const int k0 = DIR == 0 ? (r + G) * WX + i : r * WX + i + G;  // first stencil cell
+    const int p0 = r * PD + i;
+    const int ka = k0 + 2 * ST, kb = ka + ST;
+    const Roe32Shear o = roe32_2d(s_uin[ka], s_n[ka], s_t[ka], s_H[ka], s_uin[kb], s_n[kb], s_t[kb], s_H[kb], gm1);
+    Proj32Shear pf, pu;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      float d[4][5];
+      float4 h[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        float2 q[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          q[k] = s_pair[(4 * x + c) * ND + p0 + k * SD];
+          d[c][k] = q[k].x;
+        }
+        h[c] = high_differences(q);
+      }
+      project_stencil_2d(o, d, h, x ? pu : pf);
+    }
+    int bad = 0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      float fa[9], fb[9], ea[5], eb[5];
+      take_field_2d(s, o, pf, fa, ea);
+      take_field_2d(s, o, pu, fb, eb);
+      const float kap = (s == 0 || s == 3) ? 4.0f : 2.0f;
+      const float thr = s == 2 ? fmul(o.r.thr, o.T) : o.r.thr;  // the shear field carries rho v
+      if (!(prove_field(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(thr, kap)) && o.r.ok &&
+            screenable))
+        bad |= 1 << s;
+    }
+    if (bad == 0) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const double *f = s_fg + comp(c) * NCELL + k0, *d = s_df + c * ND + p0;
+        s_h[comp(c) * NI + it] = central_value(f[2 * ST], f[3 * ST], d[0], d[SD], d[3 * SD], d[4 * SD]);
+      }
+    } else {
+      s_list[atomicAdd(s_nl, 1)] = it | (bad << 16);
+    }
+  }
+  __syncthreads();
+  // ---- D3: the FP64 path of the listed interfaces
+  const int nl = *s_nl;
+  double* s_L = sm + TL::kL;
+  double* s_rs = sm + TL::kRs;
+  double* s_F = sm + TL::kF;
+  for (int base = 0; base < nl; base += FC) {
+    const int nc = min(nl - base, FC);
+    for (int q = tid; q < nc; q += NT) {
+      const int it = s_list[base + q] & 0xffff, r = it / nper, i = it - r * nper;
+      const int ka = (DIR == 0 ? (r + G) * WX + i : r * WX + i + G) + 2 * ST, kb = ka + ST;
+      double L[16], rs[4];
+      MATH::roe2d(DIR, sqrt(s_uin[ka]), sm[TL::kU + ka], sm[TL::kV + ka], s_H[ka], sqrt(s_uin[kb]), sm[TL::kU + kb],
+                  sm[TL::kV + kb], s_H[kb], a.gamma, L, rs);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) s_L[e * FC + q] = L[e];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s_rs[e * FC + q] = rs[e];
+    }
+    __syncthreads();
+    for (int item = tid; item < 4 * nc; item += NT) {
+      const int s = item / nc, q = item - s * nc;
+      const int en = s_list[base + q], it = en & 0xffff, r = it / nper, i = it - r * nper;
+      const int k0 = DIR == 0 ? (r + G) * WX + i : r * WX + i + G;
+      const double l[4] = {s_L[(4 * s) * FC + q], s_L[(4 * s + 1) * FC + q], s_L[(4 * s + 2) * FC + q],
+                           s_L[(4 * s + 3) * FC + q]};
+      const double al = s == 0 ? alpha[0] : (s == 1 ? alpha[1] : (s == 2 ? alpha[2] : alpha[3]));
+      double vp[6], vm[6];
+#pragma unroll
+      for (int kk = 0; kk < 6; ++kk) {
+        const int k = k0 + kk * ST;
+        const double f[4] = {s_fg[k], s_fg[NCELL + k], s_fg[2 * NCELL + k], s_fg[3 * NCELL + k]};
+        const double U[4] = {s_uin[k], s_uin[NCELL + k], s_uin[2 * NCELL + k], s_uin[3 * NCELL + k]};
+        MATH::project4(DIR, l, f, U, al, vp[kk], vm[kk]);
+      }
+      double qm[6];
+#pragma unroll
+      for (int kk = 0; kk < 6; ++kk) qm[kk] = vm[5 - kk];
+      if ((en >> (16 + s)) & 1) {
+        s_F[s * FC + q] = MATH::weno(vp, a.eps, a.alpha_R) + MATH::weno(qm, a.eps, a.alpha_R);
+      } else {  // a proven field: the central value on both sides
+        s_F[s * FC + q] = MATH::central6(vp) + MATH::central6(qm);
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < nc; q += NT) {
+      const int it = s_list[base + q] & 0xffff;
+      const double rs[4] = {s_rs[q], s_rs[FC + q], s_rs[2 * FC + q], s_rs[3 * FC + q]};
+      const double F[4] = {s_F[q], s_F[FC + q], s_F[2 * FC + q], s_F[3 * FC + q]};
+      double h[4];
+      MATH::backproject2d(DIR, rs, F, h);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) s_h[c * NI + it] = h[c];
+    }
+    __syncthreads();
+  }
+}
 
 __global__ void pack2d_kernel(const double* __restrict__ src, double* __restrict__ dst, long long nx, long long ny,
                               long long rowp, long long planep, int bxl, int bxh, int byl, int byh);
@@ -66,7 +268,7 @@ __global__ void __launch_bounds__(256) alpha2d_kernel(const double* __restrict__
     double U[4] = {u[idx], u[planep + idx], u[2 * planep + idx], u[3 * planep + idx]};
     double lx[4], ly[4], qq;
     MATH::euler2d_speeds(U, gamma, dx, dy, lx, ly, qq);
-    if (!(isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]))) flag_error(ctl, WT_ERR_NONPHYSICAL);
+    if (!finite4(U)) flag_error(ctl, WT_ERR_NONPHYSICAL);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       key_max(v[s], lx[s]);
@@ -80,8 +282,9 @@ __global__ void __launch_bounds__(256) alpha2d_kernel(const double* __restrict__
 }
 
 template <class MATH, int STAGE, int TX, int TY>
-__global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const Stage2DArgs a) {
-  using TL = Tile2D<TX, TY>;
+__global__ void __launch_bounds__(KernelTile2D<MATH, TX, TY>::NT, KernelTile2D<MATH, TX, TY>::kCtas) stage2d_kernel(const Stage2DArgs a) {
+  using TL = KernelTile2D<MATH, TX, TY>;
+  constexpr bool CENTRAL = MATH::kCentral;
   constexpr int WX = TL::WX, RY = TL::RY, NCELL = TL::NCELL, NI = TL::NI, NT = TL::NT;
   extern __shared__ __align__(16) double sm[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + TL::kBar);
@@ -89,13 +292,15 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
   double* s_u = sm + TL::kU;
   double* s_v = sm + TL::kV;
   double* s_H = sm + TL::kH;
-  double* s_sr = sm + TL::kSr;
   double* s_fg = sm + TL::kFg;
-  double* s_L = sm + TL::kL;
-  double* s_rs = sm + TL::kRs;
-  double* s_F = sm + TL::kF;
-  double* s_h = s_F;
-  double* s_red = s_L;
+  double *s_h, *s_red;
+  if constexpr (CENTRAL) {
+    s_h = sm + TL::kHf;
+    s_red = sm + TL::kRed;
+  } else {
+    s_h = sm + TL::kF;
+    s_red = sm + TL::kL;
+  }
 
   pdl_launch_dependents();
   pdl_wait();
@@ -173,13 +378,18 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
     const bool xin = (col >= G && col < G + tcx), yin = (r >= G && r < G + tcy);
     if (!xin && !yin) continue;  // corner: not on any stencil
     double U[4] = {s_uin[k], s_uin[NCELL + k], s_uin[2 * NCELL + k], s_uin[3 * NCELL + k]};
-    if (!(isfinite(U[0]) && isfinite(U[1]) && isfinite(U[2]) && isfinite(U[3]))) flag_error(ctl, WT_ERR_NONPHYSICAL);
-    double f[4], g[4], u, v, H, sr;
-    MATH::euler2d_cell(U, a.gamma, f, g, u, v, H, sr);
+    if (!finite4(U)) flag_error(ctl, WT_ERR_NONPHYSICAL);
+    double f[4], u, v, H;
+    if constexpr (CENTRAL) {
+      MATH::euler2d_cell_flux(U, a.gamma, f, u, v, H);
+    } else {
+      double g[4], sr;
+      MATH::euler2d_cell(U, a.gamma, f, g, u, v, H, sr);
+      sm[TL::kSr + k] = sr;
+    }
     s_u[k] = u;
     s_v[k] = v;
     s_H[k] = H;
-    s_sr[k] = sr;
     if (yin) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) s_fg[c * NCELL + k] = f[c];
@@ -187,13 +397,17 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
   }
   __syncthreads();
 
+  if constexpr (CENTRAL) {
+    central_sweep<MATH, 0, TL, TX>(a, tcx, tcy, ax, sm);
+  } else {
+    double *s_L = sm + TL::kL, *s_rs = sm + TL::kRs, *s_F = sm + TL::kF;
   // ---- x sweep.  Interface i of row r sits between cells (r+3, i+2) and (r+3, i+3).
   const int nix = (tcx + 1) * tcy;
   for (int it = tid; it < nix; it += NT) {
     const int r = it / (tcx + 1), i = it - r * (tcx + 1);
     const int ka = (r + G) * WX + i + 2, kb = ka + 1;
     double L[16], rs[4];
-    MATH::roe2d(0, s_sr[ka], s_u[ka], s_v[ka], s_H[ka], s_sr[kb], s_u[kb], s_v[kb], s_H[kb], a.gamma, L, rs);
+    MATH::roe2d(0, sm[TL::kSr + ka], s_u[ka], s_v[ka], s_H[ka], sm[TL::kSr + kb], s_u[kb], s_v[kb], s_H[kb], a.gamma, L, rs);
 #pragma unroll
     for (int e = 0; e < 16; ++e) s_L[e * NI + it] = L[e];
 #pragma unroll
@@ -230,6 +444,7 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
 #pragma unroll
     for (int c = 0; c < 4; ++c) s_h[c * NI + it] = h[c];
   }
+  }
   for (int q = tid; q < rows * tcx; q += NT) {
     const int r = q / tcx, k = r * WX + G + (q - r * tcx);
     const double U[4] = {s_uin[k], s_uin[NCELL + k], s_uin[2 * NCELL + k], s_uin[3 * NCELL + k]};
@@ -249,13 +464,17 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
     for (int c = 0; c < 4; ++c) Lx[c] = MATH::flux_diff(s_h[c * NI + it + 1], s_h[c * NI + it], a.dx, a.inv_dx);
   }
 
+  if constexpr (CENTRAL) {
+    central_sweep<MATH, 1, TL, TX>(a, tcx, tcy, ay, sm);
+  } else {
+    double *s_L = sm + TL::kL, *s_rs = sm + TL::kRs, *s_F = sm + TL::kF;
   // ---- y sweep.  Interface j of column t sits between cells (j+2, t+3) and (j+3, t+3).
   const int niy = tcx * (tcy + 1);
   for (int it = tid; it < niy; it += NT) {
     const int j = it / tcx, t = it - j * tcx;
     const int ka = (j + 2) * WX + t + G, kb = ka + WX;
     double L[16], rs[4];
-    MATH::roe2d(1, s_sr[ka], s_u[ka], s_v[ka], s_H[ka], s_sr[kb], s_u[kb], s_v[kb], s_H[kb], a.gamma, L, rs);
+    MATH::roe2d(1, sm[TL::kSr + ka], s_u[ka], s_v[ka], s_H[ka], sm[TL::kSr + kb], s_u[kb], s_v[kb], s_H[kb], a.gamma, L, rs);
 #pragma unroll
     for (int e = 0; e < 16; ++e) s_L[e * NI + it] = L[e];
 #pragma unroll
@@ -291,11 +510,15 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
     for (int c = 0; c < 4; ++c) s_h[c * NI + it] = h[c];
   }
   __syncthreads();
+  }
 
   // ---- E: L = Lx + Ly, RK combine, ghost images, wave speeds of the new state
   unsigned long long vmax[8], qmax = 0ull;
 #pragma unroll
   for (int s = 0; s < 8; ++s) vmax[s] = 0ull;
+  [[maybe_unused]] bool ok32 = false;
+  [[maybe_unused]] float l32[7] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  [[maybe_unused]] const float g32 = f32_hi(a.gamma * (a.gamma - 1.0)), idx32 = f32_hi(a.inv_dx), idy32 = f32_hi(a.inv_dy);
   if (tid < tcx * tcy) {
     const int r = tid / tcx, t = tid - r * tcx;
     const long long x = x0 + t, y = y0 + r;
@@ -348,19 +571,90 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
           if (a.bcy_hi == WT_BC_REFLECTIVE && y >= ny - G) o[(2 * ny + 2 - y) * a.rowp + col] = vy;
         }
       }
-      if (!(isfinite(uo[0]) && isfinite(uo[1]) && isfinite(uo[2]) && isfinite(uo[3])))
+      if (!finite4(uo))
         flag_error(ctl, WT_ERR_NONPHYSICAL);
-      double lx[4], ly[4], q;
-      MATH::euler2d_speeds(uo, a.gamma, a.dx, a.dy, lx, ly, q);
+      if constexpr (CENTRAL) {
+        // the output back to the tile, for the FP64 speeds of the cells that can hold a maximum
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        key_max(vmax[s], lx[s]);
-        key_max(vmax[4 + s], ly[s]);
+        for (int c = 0; c < 4; ++c) s_uin[c * NCELL + kc] = uo[c];
+        ok32 = euler2d_speeds_screen(uo, g32, idx32, idy32, l32);
+      } else {
+        double lx[4], ly[4], q;
+        MATH::euler2d_speeds(uo, a.gamma, a.dx, a.dy, lx, ly, q);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          key_max(vmax[s], lx[s]);
+          key_max(vmax[4 + s], ly[s]);
+        }
+        key_max(qmax, q);
       }
-      key_max(qmax, q);
     }
   }
-  if (STAGE != STAGE_RHS) {
+  if constexpr (CENTRAL && STAGE != STAGE_RHS) {
+    // As in 1D (the stage tiles' kScreen): the FP64 speeds (two divisions, a square root) only of
+    // the cells whose FP32 speeds come within twice their error of a tile maximum (2^-12 of the
+    // larger acoustic speed, 2^-16 of |u| or |v|, 2^-12 of q), one cell per run of bitwise-equal
+    // states, gathered from the tile into full warps: 45 FP64 instructions per cell are left
+    // to a few cells.
+    float* s_lm = reinterpret_cast<float*>(s_red);  // [7][8] warp maxima
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_red + 32);  // [9]
+    int* s_list = reinterpret_cast<int*>(sm + TL::kList);
+    int* s_nl = s_list + TL::NI;
+    const bool cell = tid < tcx * tcy;
+#pragma unroll
+    for (int f = 0; f < 7; ++f) {
+      // (non-negative floats order like their bit patterns)
+      const unsigned v = __reduce_max_sync(0xffffffffu, (cell && ok32) ? __float_as_uint(l32[f]) : 0u);
+      if ((tid & 31) == 0) s_lm[f * 8 + (tid >> 5)] = __uint_as_float(v);
+    }
+    if (tid < 9) s_key[tid] = 0ull;
+    if (tid == 0) *s_nl = 0;
+    __syncthreads();
+    if (cell) {
+      float tm[7];
+#pragma unroll
+      for (int f = 0; f < 7; ++f) {
+        tm[f] = 0.0f;
+#pragma unroll
+        for (int w = 0; w < TL::NT / 32; ++w) tm[f] = fmaxf(tm[f], s_lm[f * 8 + w]);
+      }
+      const float sx = 0x1p-12f * fmaxf(tm[0], tm[2]), sy = 0x1p-12f * fmaxf(tm[3], tm[5]);
+      bool take = !ok32 || l32[0] >= tm[0] - sx || l32[2] >= tm[2] - sx || l32[3] >= tm[3] - sy ||
+                  l32[5] >= tm[5] - sy || l32[6] >= tm[6] * (1.0f - 0x1p-12f) ||
+                  (l32[1] > 0.0f && l32[1] >= tm[1] * (1.0f - 0x1p-16f)) ||
+                  (l32[4] > 0.0f && l32[4] >= tm[4] * (1.0f - 0x1p-16f));
+      const int r = tid / tcx, t = tid - r * tcx, kc = (r + G) * WX + t + G;
+      if (take && t > 0) {  // the same state as the left neighbour's: the same speeds
+        bool dup = true;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          dup = dup && __double_as_longlong(s_uin[c * NCELL + kc]) == __double_as_longlong(s_uin[c * NCELL + kc - 1]);
+        take = !dup;
+      }
+      if (take) s_list[atomicAdd(s_nl, 1)] = kc;
+    }
+    __syncthreads();
+    for (int e = tid; e < *s_nl; e += NT) {
+      const int kc = s_list[e];
+      const double U[4] = {s_uin[kc], s_uin[NCELL + kc], s_uin[2 * NCELL + kc], s_uin[3 * NCELL + kc]};
+      double lx[4], ly[4], q;
+      MATH::euler2d_speeds(U, a.gamma, a.dx, a.dy, lx, ly, q);
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        atomicMax(&s_key[s], speed_key(lx[s]));
+        atomicMax(&s_key[4 + s], speed_key(ly[s]));
+      }
+      atomicMax(&s_key[8], speed_key(q));
+    }
+    __syncthreads();
+    constexpr int nxt = (STAGE + 1) % 3;
+    if (tid < 8) atomicMax(&ctl->amax[nxt][tid], s_key[tid]);
+    if (tid == 8) atomicMax(&ctl->cfl2d[nxt], s_key[8]);
+    if (STAGE == STAGE_RK3 && first_tile && tid == 0) {
+      ctl->t = ctl->t + dt;
+      ctl->steps = ctl->steps + 1;
+    }
+  } else if (STAGE != STAGE_RHS) {
     const int nxt = (STAGE + 1) % 3;
     block_max_atomic<8>(vmax, s_red, ctl->amax[nxt]);
     unsigned long long qa[1] = {qmax};
@@ -372,21 +666,21 @@ __global__ void __launch_bounds__(Tile2D<TX, TY>::NT, 2) stage2d_kernel(const St
   }
 }
 
-template <class MATH, int STAGE>
+template <class MATH, int STAGE, int TX>
 cudaError_t launch_stage2d_t(const Stage2DArgs& a, cudaStream_t st) {
-  constexpr int TX = 32, TY = 8;
-  using TL = Tile2D<TX, TY>;
+  constexpr int TY = kTileY<MATH>;
+  using TL = KernelTile2D<MATH, TX, TY>;
   auto kern = stage2d_kernel<MATH, STAGE, TX, TY>;  // prepare_stage2d_policy() raised its shared-memory limit
   dim3 grid((unsigned)((a.nx + TX - 1) / TX), (unsigned)((a.ny + TY - 1) / TY));
   return launch_pdl(kern, grid, dim3(TL::NT), TL::bytes, st, a);
 }
 
-template <class MATH>
-cudaError_t prepare_stage2d_policy() {
-  constexpr int TX = 32, TY = 8;
-  using TL = Tile2D<TX, TY>;
+template <class MATH, int TX>
+cudaError_t prepare_stage2d_tile() {
+  constexpr int TY = kTileY<MATH>;
+  using TL = KernelTile2D<MATH, TX, TY>;
   cudaError_t e = cudaSuccess;
-  // the tile's shared memory, and the largest carveout, so that two CTAs fit on an SM
+  // the tile's shared memory, and the largest carveout, so that kCtas CTAs fit on an SM
   const void* kerns[4] = {(const void*)stage2d_kernel<MATH, STAGE_RK1, TX, TY>,
                           (const void*)stage2d_kernel<MATH, STAGE_RK2, TX, TY>,
                           (const void*)stage2d_kernel<MATH, STAGE_RK3, TX, TY>,
@@ -400,12 +694,38 @@ cudaError_t prepare_stage2d_policy() {
 }
 
 template <class MATH>
+cudaError_t prepare_stage2d_policy() {
+  cudaError_t e = prepare_stage2d_tile<MATH, 32>();
+  if constexpr (MATH::kCentral) {
+    if (e == cudaSuccess) e = prepare_stage2d_tile<MATH, 16>();
+  }
+  return e;
+}
+
+// Width of the tiles (central): 32 columns (two CTAs of 256 threads per SM) on large grids, whose halo is
+// the smaller share; 16 (four of 128) where 32-column tiles make fewer than four waves of the
+// GPU's 304 slots, since the tiles on a front cost several times the others and smaller ones
+// spread them (120 x 360: 16.8 -> 13.6 ms for 40 steps; 2048 x 2048: 18.1 -> 19.3 ms for 2).
+template <class MATH>
+bool narrow_tiles(const Stage2DArgs& a) {
+  return MATH::kCentral && ((a.nx + 31) / 32) * ((a.ny + kTileY<MATH> - 1) / kTileY<MATH>) < 4 * 304;
+}
+
+template <class MATH, int STAGE>
+cudaError_t launch_stage2d_w(const Stage2DArgs& a, cudaStream_t st) {
+  if constexpr (MATH::kCentral) {
+    if (narrow_tiles<MATH>(a)) return launch_stage2d_t<MATH, STAGE, 16>(a, st);
+  }
+  return launch_stage2d_t<MATH, STAGE, 32>(a, st);
+}
+
+template <class MATH>
 cudaError_t launch_stage2d_policy(int stage, const Stage2DArgs& a, cudaStream_t st) {
   switch (stage) {
-    case STAGE_RK1: return launch_stage2d_t<MATH, STAGE_RK1>(a, st);
-    case STAGE_RK2: return launch_stage2d_t<MATH, STAGE_RK2>(a, st);
-    case STAGE_RK3: return launch_stage2d_t<MATH, STAGE_RK3>(a, st);
-    case STAGE_RHS: return launch_stage2d_t<MATH, STAGE_RHS>(a, st);
+    case STAGE_RK1: return launch_stage2d_w<MATH, STAGE_RK1>(a, st);
+    case STAGE_RK2: return launch_stage2d_w<MATH, STAGE_RK2>(a, st);
+    case STAGE_RK3: return launch_stage2d_w<MATH, STAGE_RK3>(a, st);
+    case STAGE_RHS: return launch_stage2d_w<MATH, STAGE_RHS>(a, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -55,11 +55,22 @@ struct FastMath {
     double ir;
     euler_cell_ir(U, gamma, f, u, H, sr, p, ir);
   }
+  // 1 / x for the central tiles' cells: the hardware's approximation (the FP64 pipe takes no part in it) and
+  // one step of Halley's iteration, y (1 + e + e^2) with e = 1 - x y, which cubes the error: three
+  // FP64 instructions instead of the five or six of a correctly rounded reciprocal, within
+  // 2^-52.  Magnitudes outside [2^-1000, 2^1000] (and NaN, inf) take the division.
+  __device__ __forceinline__ static double recip(double x) {
+    if ((unsigned)(exp_mag(x) - 0x01700000) >= 0x7d000000u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+  }
   // the central tiles' cell quantities (wt_central.cuh): f, u and H; sqrt(rho) is taken only where an
   // interface needs Roe's average in FP64
   static constexpr bool kCentral = true;
   __device__ __forceinline__ static void euler_cell_flux(const double* U, double gamma, double* f, double& u, double& H) {
-    const double ir = 1.0 / U[0];
+    const double ir = recip(U[0]);
     u = __dmul_rn(U[1], ir);
     const double p = __dmul_rn(gamma - 1.0, fma(-0.5 * U[1], u, U[2]));
     const double e = __dadd_rn(U[2], p);
@@ -258,6 +269,11 @@ struct FastMath {
     const double c3 = theta1 ? -3.0 / 60.0 : -7.0 / 60.0;
     const double c4 = theta1 ? 0.0 : 1.0 / 60.0;
     return fma(c4, d4, fma(c3, d3, fma(c2, d2, fma(c1, d1, c0 * d0)))) + q2;
+  }
+
+  // the restricted stencil with theta = 0, from its cell values
+  __device__ __forceinline__ static double central6(const double* q) {
+    return linear_theta(q[1] - q[0], q[2] - q[1], q[3] - q[2], q[4] - q[3], q[5] - q[4], q[2], false);
   }
 
   // |x| as the high word of its bit pattern (orders like |x| for finite x; inf and NaN top it)
@@ -568,6 +584,20 @@ struct FastMath {
     g[3] = e * v;
     H = e * ir;
     sr = sqrt(U[0]);
+  }
+  // the central tiles' cell quantities: those of euler2d_cell without sqrt(rho)
+  __device__ __forceinline__ static void euler2d_cell_flux(const double* U, double gamma, double* f, double& u,
+                                                           double& v, double& H) {
+    const double ir = recip(U[0]);
+    u = __dmul_rn(U[1], ir);
+    v = __dmul_rn(U[2], ir);
+    const double p = __dmul_rn(gamma - 1.0, fma(-0.5, dot2(U[1], u, U[2], v), U[3]));
+    const double e = __dadd_rn(U[3], p);
+    f[0] = U[1];
+    f[1] = fma(U[1], u, p);
+    f[2] = __dmul_rn(U[1], v);
+    f[3] = __dmul_rn(e, u);
+    H = __dmul_rn(e, ir);
   }
   // g of euler2d_cell alone, from the u and v it returned (the same operations; p and e are
   // rounded explicitly in both, so that neither is contracted differently at either site)

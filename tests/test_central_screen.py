@@ -263,3 +263,40 @@ def test_screened_paths_match_the_oracle_and_each_other(wtlib, oracle, kind, n, 
         runs.append(u.cpu().numpy())
     for r in runs[1:]:
         assert np.array_equal(r, runs[0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["front", "smooth", "noise", "large values"])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (7, 16), (15, 8), (16, 7), (17, 15), (33, 6), (64, 29), (224, 1260)])
+def test_screened_2d_matches_the_oracle(wtlib, oracle, kind, nx, ny):
+    """Edges of the 16 x 7 tiles, and a grid of 32 x 7 ones: RHS as above, and one step's maxima (the next
+    step's dt) equal to those of the speeds of every cell."""
+    b, O = wtlib, oracle
+    x, y = np.meshgrid((np.arange(nx) + 0.5) / nx, (np.arange(ny) + 0.5) / ny)
+    wave = 1 + 0.2 * np.sin(2 * np.pi * (x + 2 * y))
+    one = np.ones((ny, nx))
+    scale = 2.0**62 if kind == "large values" else 1.0
+    if kind == "front":
+        U = W.cons_2d(np.where(x + y > 0.8, 1.0, 0.125), 0.3 * wave, 0.1 * one, np.where(x + y > 0.8, 1.0, 0.1))
+    elif kind == "noise":
+        U = W.ulp_perturbed(W.cons_2d(0.7 * one, 0.3 * one, 0.2 * one, 0.9 * one), 5)
+    else:
+        U = W.cons_2d(wave * scale, 0.4 + 0.1 * np.cos(2 * np.pi * y), 0.2 * wave, wave * scale)
+    dx, dy = 1.0 / nx, 1.0 / ny
+    P = O.problem(O.FLUX_EULER2D, bc=0, alpha_R=10.0)
+    ref = O.rhs(P, U, dx, dy)
+    spread = np.max([np.abs(O.rhs(P, W.ulp_perturbed(U, s), dx, dy) - ref).max(axis=(1, 2)) for s in range(3)], axis=0)
+    tol = np.maximum(1e-13 * np.abs(ref).max(axis=(1, 2)), 10 * spread)
+    g = b.grid_2d(nx, ny)
+    prob = b.problem(b.WT_FLUX_EULER2D, alpha_R=10.0)
+    ws = b.alloc_workspace(b.workspace_bytes(prob, g))
+    u = torch.from_numpy(np.ascontiguousarray(U)).cuda()
+    L = torch.empty_like(u)
+    b.weno_theta_rhs(prob, g, u, L, ws)
+    assert np.all(np.abs(L.cpu().numpy() - ref).max(axis=(1, 2)) <= tol)
+    # two steps in one call, and in two: the second call takes the speeds of every cell (alpha2d)
+    v, w = u.clone(), u.clone()
+    t2, _ = b.weno_theta_step(prob, g, v, 0.4, ws, max_steps=2)
+    ta, _ = b.weno_theta_step(prob, g, w, 0.4, ws, max_steps=1)
+    tb, _ = b.weno_theta_step(prob, g, w, 0.4, ws, max_steps=1)
+    assert torch.equal(v, w) and t2 == ta + tb
