@@ -18,9 +18,9 @@
 // Every operation is an explicit rounded intrinsic: all kernels take the same decisions.
 //
 // Measured (1D, GB300): FP64 thread instructions per cell and stage 364 -> about 60 where the data are
-// smooth; a run of 999,983 cells 17.96 -> 5.32 ms for 8 steps, a batch of 12.0 M cells in problems of
-// 256 to 65536 cells 103.4 -> 30.6 ms for 4 steps, 600 problems of 64 to 1024 cells (a third of
-// the interfaces listed) 14.0 -> 12.7 ms for 20 steps.  Error of L against extended precision:
+// smooth; a run of 999,983 cells 18.0 -> 4.5 ms for 8 steps, a batch of 12.0 M cells in problems of
+// 256 to 65536 cells 103.6 -> 29.0 ms for 4 steps, 600 problems of 64 to 1024 cells (a third of
+// the interfaces listed) 14.3 -> 12.6 ms for 20 steps.  Error of L against extended precision:
 // as before or smaller (smooth data 5.5e-14 -> 1.5e-14 rms at 5000 cells; C f rounds less).
 #pragma once
 
@@ -196,17 +196,23 @@ __device__ __forceinline__ void take_field(int s, const Roe32& r, const Proj32& 
 // One field of one interface.  a, b: the projections of the differences of f and of u: [0..4] the
 // cell differences, [5] third, [6], [7] fourth, [8] fifth; ea, eb: their error bounds ([0] for all
 // five cell differences, [1..4] for [5..8]).  al: alpha_s.  The sides' stencil differences are (a
-// +- al b) times kappa (1/4 for the acoustic fields, 1/2 for the entropy field); epsk = eps /
-// kappa^2, thrk = thr / kappa.  True only if both sides are restricted and on each theta = 0 or
-// theta does not matter.
+// +- al b) times kappa (1/4 for the acoustic fields, 1/2 for the others); epsk = eps / kappa^2,
+// thrk = thr / kappa.  Returns 0 if some decision is left to FP64; else 1, plus 2 where the +
+// side has theta = 1, plus 4 where the - side has (0 where theta does not matter).
 //   beta_k: with each difference within eta and S their maximum, the indicators move by at most 54
 //   S eta + 27 eta^2 (the worst: beta_3, forms of 1-norm 8 and 3), and their FP32 roundings by
 //   2^-16 S^2; the test is that of Eq. (be_res), max beta <= alpha_R (eps + min beta), with the
 //   indicators moved against it.
-//   theta = 0: tau6's upper bound is below tau5's lower bound (Eqs. (tau_5), (tau_6), (tau_we6)).
-__device__ __forceinline__ bool prove_field(const float* a, const float* b, const float* ea, const float* eb, float al,
-                                            float epsk, float alpha_R, float thrk) {
+//   theta = 0: tau6's upper bound is below tau5's lower bound (Eqs. (tau_5), (tau_6), (tau_we6));
+//   theta = 1: the other way round.  TH1 = false: only theta = 0 is proven (else 0).  The 2D sweeps take
+//   both verdicts (with the reduction of phase E's maxima by warps: 2048 x 2048 vortices 18.8 ->
+//   17.5 ms, 120 x 360 Rayleigh-Taylor 13.8 -> 11.6 ms); in the 1D Euler tiles the second one's
+//   registers cost more than it saves (batch of 1024 problems 29.0 -> 30.0 .. 32.9 ms).
+template <bool TH1 = true>
+__device__ __forceinline__ int prove_field(const float* a, const float* b, const float* ea, const float* eb, float al,
+                                            float epsk, float alpha_R, float thrk, int sides = 3) {
   constexpr float F1312 = 13.0f / 12.0f, F1348 = 13.0f / 48.0f;
+  int verdict = 1;
   bool ok = true;
   float bm = fmaxf(fmaxf(fmaxf(fabsf(b[0]), fabsf(b[1])), fmaxf(fabsf(b[2]), fabsf(b[3]))), fabsf(b[4]));
   const float eta = ffma(al, ffma(0x1p-21f, bm, eb[0]), ea[0]);
@@ -215,6 +221,7 @@ __device__ __forceinline__ bool prove_field(const float* a, const float* b, cons
   for (int v = 0; v < 4; ++v) ehi[v] = ffma(al, ffma(0x1p-21f, fabsf(b[5 + v]), eb[1 + v]), ea[1 + v]);
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
+    if (!((sides >> side) & 1)) continue;  // (a side known to vanish)
     const float sa = side ? -al : al;
     float d[5];
 #pragma unroll
@@ -236,15 +243,44 @@ __device__ __forceinline__ bool prove_field(const float* a, const float* b, cons
     const int y = side ? 7 : 6, z = side ? 6 : 7;  // the side's own fourth difference, the other
     const float t3 = fabsf(ffma(sa, b[5], a[5]));
     const float ty = ffma(sa, b[y], a[y]), tz = ffma(sa, b[z], a[z]);
-    const float t5 = fadd(fabsf(ffma(sa, b[8], a[8])), ehi[3]);
+    const float a5 = fabsf(ffma(sa, b[8], a[8])), a6 = fabsf(fadd(ty, tz)), e6 = fadd(ehi[1], ehi[2]);
+    const float t5 = fadd(a5, ehi[3]), hi6 = fadd(a6, e6);
     const float lo3 = fmaxf(fsub(t3, ehi[0]), 0.0f), lo4 = fmaxf(fsub(fabsf(ty), ehi[y - 5]), 0.0f);
-    const float hi6 = fadd(fabsf(fadd(ty, tz)), fadd(ehi[1], ehi[2]));
     const float tau5lo = ffma(fmul(F1312, lo4), lo4, fmul(lo3, lo3));
     const float tau6hi = ffma(fmul(F1312, t5), t5, fmul(0.25f, fmul(hi6, hi6)));
     const bool theta0 = fmul(tau6hi, 1.0f + 0x1p-18f) < tau5lo && tau5lo > 0x1p-100f;
-    ok = ok && restricted && (theta0 || t5 <= thrk);
+    ok = ok && restricted;
+    if (!TH1) {
+      ok = ok && (theta0 || t5 <= thrk);
+    } else if (!(theta0 || t5 <= thrk)) {  // (few stencils: not evaluated for the others)
+      const float hi3 = fadd(t3, ehi[0]), hi4 = fadd(fabsf(ty), ehi[y - 5]);
+      const float lo5 = fmaxf(fsub(a5, ehi[3]), 0.0f), lo6 = fmaxf(fsub(a6, e6), 0.0f);
+      const float tau5hi = ffma(fmul(F1312, hi4), hi4, fmul(hi3, hi3));
+      const float tau6lo = ffma(fmul(F1312, lo5), lo5, fmul(0.25f, fmul(lo6, lo6)));
+      ok = ok && fmul(tau5hi, 1.0f + 0x1p-18f) < tau6lo && tau6lo > 0x1p-100f;
+      verdict |= side ? 4 : 2;
+    }
   }
-  return ok;
+  return ok ? verdict : 0;
+}
+constexpr int kAllCentral = 1 | 1 << 3 | 1 << 6;  // the verdicts of three fields, three bits each
+constexpr int kAllCentral2D = kAllCentral | 1 << 9;
+
+// the fifth difference from the five cell differences, antisymmetric for mirrored data
+__device__ __forceinline__ double fifth_difference(double d0, double d1, double d2, double d3, double d4) {
+  return fma(6.0, d2, fma(-4.0, __dadd_rn(d1, d3), __dadd_rn(d0, d4)));
+}
+// the same from the six cell values
+__device__ __forceinline__ double fifth_difference_q(double q0, double q1, double q2, double q3, double q4, double q5) {
+  return fma(10.0, __dsub_rn(q3, q2), fma(-5.0, __dsub_rn(q4, q1), __dsub_rn(q5, q0)));
+}
+// F_s of a field whose decisions the screen has taken: C v+ + C v- less the theta = 1 sides' Delta^5 v / 60
+// (the mirrored side's with the other sign), from c = l.(C f), a = l.(Delta^5 f), b = l.(Delta^5 u)
+// with l scaled by 1/2
+__device__ __forceinline__ double decided_field(int verdict, double c, double a, double b, double al) {
+  const double tp = verdict & 2 ? 1.0 : 0.0, tm = verdict & 4 ? 1.0 : 0.0;
+  const double w = fma(al * (tp + tm), b, (tp - tm) * a);
+  return fma(-1.0 / 60.0, w, 2.0 * c);
 }
 
 // ---- 2D (Sec. 4.3): normal velocity u and tangential velocity t of a sweep.  Projections with w1 = xn - u

@@ -336,7 +336,7 @@ struct Screen32 {
   float fa[9], fb[9], ea[5], eb[5];
   __device__ __forceinline__ bool prove(int s, const double (&alpha)[3], float eps, float aR) const {
     const float al = f32_trunc(s == 0 ? alpha[0] : (s == 1 ? alpha[1] : alpha[2])), kap = s == 1 ? 2.0f : 4.0f;
-    return r.ok && prove_field(fa, fb, ea, eb, al, fmul(eps, kap * kap), aR, fmul(r.thr, kap));
+    return r.ok && prove_field<false>(fa, fb, ea, eb, al, fmul(eps, kap * kap), aR, fmul(r.thr, kap));
   }
 };
 template <class TL>
@@ -684,7 +684,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
         take_field(s, r, pf, fa, ea);
         take_field(s, r, pu, fb, eb);
         const float kap = s == 1 ? 2.0f : 4.0f;
-        if (!(prove_field(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(r.thr, kap)) && r.ok &&
+        if (!(prove_field<false>(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(r.thr, kap)) && r.ok &&
               screenable))
           bad |= 1 << s;
       }

@@ -51,7 +51,7 @@ struct Tile2D {
 
 // What the fast policy's kernel costs: about 190 FP64 thread instructions per cell and stage where the data
 // are smooth (1245 with every interface projected), 58 % of the FP64 pipe's cycles at 16 warps per
-// SM; 2048 x 2048 vortices 59.8 -> 18.1 ms for two steps, 120 x 360 Rayleigh-Taylor 22.3 -> 13.6
+// SM; 2048 x 2048 vortices 59.8 -> 17.4 ms for two steps, 120 x 360 Rayleigh-Taylor 22.3 -> 11.5
 // ms for 40 (a fifth of its y interfaces are on fronts and take the FP64 path).
 //
 // Tile of the central screen (wt_central.cuh; the fast policy): no eigenvector or reconstruction
@@ -86,8 +86,10 @@ struct Tile2DC {
   static_assert(24 * FC <= 8 * ND, "the FP64 path's buffers over the pairs");
   static constexpr int kHf = kPair + 8 * ND;           // [4][NI]
   static constexpr int kRed = kHf + 4 * NI;            // maxima of the speeds
-  static constexpr int kList = kRed + 48;              // ints [NI], and a counter each for the list and the speeds
-  static constexpr int kTotal = kList + (NI + 1) / 2 + 2;
+  static constexpr int kList = kRed + 32 + 9 * (NT / 32) + (NT / 32) % 2;              // ints [NI]: listed interfaces (or cells, for the speeds)
+  static constexpr int kItems = kList + (NI + 1) / 2;  // ints [4 * FC]: (field, slot) pairs of the FP64 path
+  static constexpr int kCnt = kItems + 2 * FC;         // ints: listed, items
+  static constexpr int kTotal = kCnt + 1;
   static constexpr size_t bytes = sizeof(double) * kTotal;
   static_assert(kCtas * (bytes + 1024) <= 228 * 1024, "512 threads' tiles must fit on one SM");
 };
@@ -118,7 +120,8 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
   float2* s_pair = reinterpret_cast<float2*>(sm + TL::kPair);
   double* s_h = sm + TL::kHf;
   int* s_list = reinterpret_cast<int*>(sm + TL::kList);
-  int* s_nl = s_list + NI;
+  int* s_nl = reinterpret_cast<int*>(sm + TL::kCnt);  // listed interfaces, items of the FP64 path
+  int* s_item = reinterpret_cast<int*>(sm + TL::kItems);
   // components in the sweep's order (density, normal momentum, tangential momentum, energy)
   auto comp = [](int c) { return c == 1 ? N1 : (c == 2 ? T1 : c); };
   const int nper = DIR == 0 ? tcx + 1 : tcx;  // interfaces per row of the tile
@@ -139,7 +142,7 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
       s_pair[(4 + c) * ND + p] = f32_pair(__dsub_rn(y[ST], y[0]));
     }
   }
-  if (tid == 0) *s_nl = 0;
+  if (tid == 0) s_nl[0] = s_nl[1] = 0;
   __syncthreads();
   // ---- D2
   const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
@@ -167,7 +170,7 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
       }
       project_stencil_2d(o, d, h, x ? pu : pf);
     }
-    int bad = 0;
+    int verdicts = 0;  // three bits per field
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       float fa[9], fb[9], ea[5], eb[5];
@@ -175,18 +178,17 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
       take_field_2d(s, o, pu, fb, eb);
       const float kap = (s == 0 || s == 3) ? 4.0f : 2.0f;
       const float thr = s == 2 ? fmul(o.r.thr, o.T) : o.r.thr;  // the shear field carries rho v
-      if (!(prove_field(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(thr, kap)) && o.r.ok &&
-            screenable))
-        bad |= 1 << s;
+      const int v = prove_field(fa, fb, ea, eb, f32_trunc(alpha[s]), fmul(eps, kap * kap), aR, fmul(thr, kap));
+      verdicts |= (o.r.ok && screenable ? v : 0) << (3 * s);
     }
-    if (bad == 0) {
+    if (verdicts == kAllCentral2D) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const double *f = s_fg + comp(c) * NCELL + k0, *d = s_df + c * ND + p0;
         s_h[comp(c) * NI + it] = central_value(f[2 * ST], f[3 * ST], d[0], d[SD], d[3 * SD], d[4 * SD]);
       }
     } else {
-      s_list[atomicAdd(s_nl, 1)] = it | (bad << 16);
+      s_list[atomicAdd(s_nl, 1)] = it | (verdicts << 16);
     }
   }
   __syncthreads();
@@ -198,20 +200,50 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
   for (int base = 0; base < nl; base += FC) {
     const int nc = min(nl - base, FC);
     for (int q = tid; q < nc; q += NT) {
-      const int it = s_list[base + q] & 0xffff, r = it / nper, i = it - r * nper;
-      const int ka = (DIR == 0 ? (r + G) * WX + i : r * WX + i + G) + 2 * ST, kb = ka + ST;
+      const int it = s_list[base + q] & 0xffff, verdicts = s_list[base + q] >> 16, r = it / nper, i = it - r * nper;
+      const int k0 = DIR == 0 ? (r + G) * WX + i : r * WX + i + G, p0 = r * PD + i;
+      const int ka = k0 + 2 * ST, kb = ka + ST;
       double L[16], rs[4];
-      MATH::roe2d(DIR, sqrt(s_uin[ka]), sm[TL::kU + ka], sm[TL::kV + ka], s_H[ka], sqrt(s_uin[kb]), sm[TL::kU + kb],
-                  sm[TL::kV + kb], s_H[kb], a.gamma, L, rs);
+      MATH::roe2d(DIR, MATH::sqrt_rho(s_uin[ka]), sm[TL::kU + ka], sm[TL::kV + ka], s_H[ka], MATH::sqrt_rho(s_uin[kb]),
+                  sm[TL::kU + kb], sm[TL::kV + kb], s_H[kb], a.gamma, L, rs);
 #pragma unroll
       for (int e = 0; e < 16; ++e) s_L[e * FC + q] = L[e];
 #pragma unroll
       for (int e = 0; e < 4; ++e) s_rs[e * FC + q] = rs[e];
+      int un = 0;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) un |= ((verdicts >> (3 * s)) & 7) == 0 ? 1 << s : 0;
+      if (un != 15) {  // the fields the screen has decided (decided_field)
+        double C[4], A[4], B[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {  // in the sweep's order of components
+          const double *f = s_fg + comp(c) * NCELL + k0, *v = s_uin + comp(c) * NCELL + k0, *x = s_df + c * ND + p0;
+          C[c] = central_value(f[2 * ST], f[3 * ST], x[0], x[SD], x[3 * SD], x[4 * SD]);
+          A[c] = fifth_difference(x[0], x[SD], x[2 * SD], x[3 * SD], x[4 * SD]);
+          B[c] = fifth_difference_q(v[0], v[ST], v[2 * ST], v[3 * ST], v[4 * ST], v[5 * ST]);
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          if ((un >> s) & 1) continue;
+          const double l[4] = {L[4 * s], L[4 * s + N1], L[4 * s + T1], L[4 * s + 3]};
+          const double c = fma(l[3], C[3], fma(l[2], C[2], fma(l[1], C[1], l[0] * C[0])));
+          const double p = fma(l[3], A[3], fma(l[2], A[2], fma(l[1], A[1], l[0] * A[0])));
+          const double w = fma(l[3], B[3], fma(l[2], B[2], fma(l[1], B[1], l[0] * B[0])));
+          s_F[s * FC + q] = decided_field((verdicts >> (3 * s)) & 7, c, p, w, alpha[s]);
+        }
+      }
+      if (un != 0) {
+        int at = atomicAdd(&s_nl[1], __popc(un));
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+          if ((un >> s) & 1) s_item[at++] = q | (s << 16);
+      }
     }
     __syncthreads();
-    for (int item = tid; item < 4 * nc; item += NT) {
-      const int s = item / nc, q = item - s * nc;
-      const int en = s_list[base + q], it = en & 0xffff, r = it / nper, i = it - r * nper;
+    const int nit = s_nl[1];
+    for (int e = tid; e < nit; e += NT) {
+      const int s = s_item[e] >> 16, q = s_item[e] & 0xffff;
+      const int it = s_list[base + q] & 0xffff, r = it / nper, i = it - r * nper;
       const int k0 = DIR == 0 ? (r + G) * WX + i : r * WX + i + G;
       const double l[4] = {s_L[(4 * s) * FC + q], s_L[(4 * s + 1) * FC + q], s_L[(4 * s + 2) * FC + q],
                            s_L[(4 * s + 3) * FC + q]};
@@ -227,11 +259,7 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
       double qm[6];
 #pragma unroll
       for (int kk = 0; kk < 6; ++kk) qm[kk] = vm[5 - kk];
-      if ((en >> (16 + s)) & 1) {
-        s_F[s * FC + q] = MATH::weno(vp, a.eps, a.alpha_R) + MATH::weno(qm, a.eps, a.alpha_R);
-      } else {  // a proven field: the central value on both sides
-        s_F[s * FC + q] = MATH::central6(vp) + MATH::central6(qm);
-      }
+      s_F[s * FC + q] = MATH::weno(vp, a.eps, a.alpha_R) + MATH::weno(qm, a.eps, a.alpha_R);
     }
     __syncthreads();
     for (int q = tid; q < nc; q += NT) {
@@ -243,6 +271,7 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
 #pragma unroll
       for (int c = 0; c < 4; ++c) s_h[c * NI + it] = h[c];
     }
+    if (tid == 0) s_nl[1] = 0;
     __syncthreads();
   }
 }
@@ -597,9 +626,9 @@ __global__ void __launch_bounds__(KernelTile2D<MATH, TX, TY>::NT, KernelTile2D<M
     // states, gathered from the tile into full warps: 45 FP64 instructions per cell are left
     // to a few cells.
     float* s_lm = reinterpret_cast<float*>(s_red);  // [7][8] warp maxima
-    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_red + 32);  // [9]
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_red + 32);  // [warps][9]
     int* s_list = reinterpret_cast<int*>(sm + TL::kList);
-    int* s_nl = s_list + TL::NI;
+    int* s_nl = reinterpret_cast<int*>(sm + TL::kCnt);
     const bool cell = tid < tcx * tcy;
 #pragma unroll
     for (int f = 0; f < 7; ++f) {
@@ -607,7 +636,6 @@ __global__ void __launch_bounds__(KernelTile2D<MATH, TX, TY>::NT, KernelTile2D<M
       const unsigned v = __reduce_max_sync(0xffffffffu, (cell && ok32) ? __float_as_uint(l32[f]) : 0u);
       if ((tid & 31) == 0) s_lm[f * 8 + (tid >> 5)] = __uint_as_float(v);
     }
-    if (tid < 9) s_key[tid] = 0ull;
     if (tid == 0) *s_nl = 0;
     __syncthreads();
     if (cell) {
@@ -634,22 +662,36 @@ __global__ void __launch_bounds__(KernelTile2D<MATH, TX, TY>::NT, KernelTile2D<M
       if (take) s_list[atomicAdd(s_nl, 1)] = kc;
     }
     __syncthreads();
-    for (int e = tid; e < *s_nl; e += NT) {
-      const int kc = s_list[e];
-      const double U[4] = {s_uin[kc], s_uin[NCELL + kc], s_uin[2 * NCELL + kc], s_uin[3 * NCELL + kc]};
-      double lx[4], ly[4], q;
-      MATH::euler2d_speeds(U, a.gamma, a.dx, a.dy, lx, ly, q);
+    const int nsp = *s_nl;
+    {
+      unsigned long long key[9] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+      if (tid < nsp) {  // (at most one cell per thread)
+        const int kc = s_list[tid];
+        const double U[4] = {s_uin[kc], s_uin[NCELL + kc], s_uin[2 * NCELL + kc], s_uin[3 * NCELL + kc]};
+        double lx[4], ly[4], q;
+        MATH::euler2d_speeds(U, a.gamma, a.dx, a.dy, lx, ly, q);
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        atomicMax(&s_key[s], speed_key(lx[s]));
-        atomicMax(&s_key[4 + s], speed_key(ly[s]));
+        for (int s = 0; s < 4; ++s) {
+          key[s] = speed_key(lx[s]);
+          key[4 + s] = speed_key(ly[s]);
+        }
+        key[8] = speed_key(q);
       }
-      atomicMax(&s_key[8], speed_key(q));
+      if ((tid & ~31) < nsp) {
+#pragma unroll
+        for (int f = 0; f < 9; ++f) {
+          const unsigned long long m = warp_max_key_redux(key[f]);
+          if ((tid & 31) == 0) s_key[9 * (tid >> 5) + f] = m;
+        }
+      }
     }
     __syncthreads();
     constexpr int nxt = (STAGE + 1) % 3;
-    if (tid < 8) atomicMax(&ctl->amax[nxt][tid], s_key[tid]);
-    if (tid == 8) atomicMax(&ctl->cfl2d[nxt], s_key[8]);
+    if (tid < 9) {
+      unsigned long long m = 0ull;
+      for (int w = 0; 32 * w < nsp; ++w) m = max(m, s_key[9 * w + tid]);
+      atomicMax(tid < 8 ? &ctl->amax[nxt][tid] : &ctl->cfl2d[nxt], m);
+    }
     if (STAGE == STAGE_RK3 && first_tile && tid == 0) {
       ctl->t = ctl->t + dt;
       ctl->steps = ctl->steps + 1;

@@ -1,9 +1,10 @@
 """The central screen of the fast policy's 1D Euler tiles (wt_central.cuh).
 
-An interface takes the central flux C f only where FP32 proves, for all three fields and both
-sides, that the reconstruction is restricted (Eq. (be_res)) and that theta = 0 (Eq. (tau_we6)) or
-|Delta^5 v| / 60 is at most 2^-53 rho (|u| + c).  ``screen`` restates that proof in numpy float32, step
-by step as the kernels take it; the CPU test holds every proven field against the decisions in
+A field of an interface is decided in FP32 only where that proves, on both sides, that the
+reconstruction is restricted (Eq. (be_res)) and either theta (Eq. (tau_we6)) or that |Delta^5 v| / 60 is at
+most 2^-53 rho (|u| + c), where theta does not matter; an interface takes the central flux C f
+where all fields have theta = 0 so.  ``screen`` restates that proof in numpy float32, step by step
+as the kernels take it; the CPU test holds every decided field against the decisions in
 extended precision.  The GPU tests hold the kernels against the oracle, and every launch
 path against the others bit for bit, on data at the screen's edges."""
 import numpy as np
@@ -42,7 +43,8 @@ def _high(d):
 
 
 def screen(f, U, vel, H, al, eps, aR):
-    """proven[field][interface] from six-cell windows f, U [3][6][n] (float64), and the two centre cells'
+    """Verdicts [field][interface] (0: left to FP64; else 1, + 2 if the + side has theta = 1, + 4 if the - side
+    has) from six-cell windows f, U [3][6][n] (float64), and the two centre cells'
     velocity and enthalpy."""
     with np.errstate(all="ignore"):
         r0, r1 = _trunc(U[0, 2]), _trunc(U[0, 3])
@@ -104,7 +106,7 @@ def screen(f, U, vel, H, al, eps, aR):
             bm = np.max([np.abs(A[1][k]) for k in range(5)], axis=0)
             eta = a * (f4(2.0**-21) * bm + E[1][0]) + E[0][0]
             eh = [a * (f4(2.0**-21) * np.abs(A[1][5 + v]) + E[1][1 + v]) + E[0][1 + v] for v in range(4)]
-            good = ok.copy()
+            good, verdict = ok.copy(), np.ones(ok.shape, dtype=int)
             C, C3 = f4(13 / 12), f4(13 / 48)
             for side in range(2):
                 sa_ = -a if side else a
@@ -119,14 +121,21 @@ def screen(f, U, vel, H, al, eps, aR):
                 y, z = (7, 6) if side else (6, 7)
                 t3 = np.abs(sa_ * A[1][5] + A[0][5])
                 ty, tz = sa_ * A[1][y] + A[0][y], sa_ * A[1][z] + A[0][z]
-                t5 = np.abs(sa_ * A[1][8] + A[0][8]) + eh[3]
+                a5, a6, e6 = np.abs(sa_ * A[1][8] + A[0][8]), np.abs(ty + tz), eh[1] + eh[2]
+                t5, lo5 = a5 + eh[3], np.maximum(a5 - eh[3], 0)
+                hi3, hi4, lo6 = t3 + eh[0], np.abs(ty) + eh[y - 5], np.maximum(a6 - e6, 0)
                 lo3, lo4 = np.maximum(t3 - eh[0], 0), np.maximum(np.abs(ty) - eh[y - 5], 0)
-                hi6 = np.abs(ty + tz) + (eh[1] + eh[2])
+                hi6 = a6 + e6
                 t5lo = C * lo4 * lo4 + lo3 * lo3
                 t6hi = C * t5 * t5 + f4(0.25) * (hi6 * hi6)
                 theta0 = (t6hi * f4(1 + 2.0**-18) < t5lo) & (t5lo > f4(2.0**-100))
-                good &= restricted & (theta0 | (t5 <= thr * kap))
-            out.append(good)
+                t5hi = C * hi4 * hi4 + hi3 * hi3
+                t6lo = C * lo5 * lo5 + f4(0.25) * (lo6 * lo6)
+                theta1 = (t5hi * f4(1 + 2.0**-18) < t6lo) & (t6lo > f4(2.0**-100))
+                zero = theta0 | (t5 <= thr * kap)
+                good &= restricted & (zero | theta1)
+                verdict[~zero] |= 4 if side else 2
+            out.append(np.where(good, verdict, 0))
         return np.array(out)
 
 
@@ -185,8 +194,8 @@ def _states():
 
 
 @pytest.mark.parametrize("aR", [1.0, 10.0, 50.0])
-def test_every_proven_field_is_central(aR):
-    eps, shown = 1e-10, 0
+def test_every_decided_field_is_as_decided(aR):
+    eps, central, upwind = 1e-10, 0, 0
     for U in _states():
         f, u, H, c = _fields(U)
         n = U.shape[1] - 5
@@ -198,11 +207,14 @@ def test_every_proven_field_is_central(aR):
         for s in range(3):
             for side in range(2):
                 restricted, gap, d5 = res[2 * s + side]
-                assert np.all(restricted[ok[s]])
+                decided, one = ok[s] != 0, (ok[s] & (4 if side else 2)) != 0
+                assert np.all(restricted[decided])
                 free = d5 <= 60 * np.longdouble(2.0)**-53 * scale
-                assert np.all((gap < 0)[ok[s]] | free[ok[s]])
-        shown += int(ok.all(axis=0).sum())
-    assert shown > 20000  # the screen proves most of the smooth data
+                assert np.all(((gap < 0) | free)[decided & ~one])
+                assert np.all((gap > 0)[one])
+                upwind += int(one.sum())
+        central += int((ok == 1).all(axis=0).sum())
+    assert central > 20000 and upwind > 0  # the screen decides most of the smooth data, both ways
 
 
 torch = pytest.importorskip("torch")
