@@ -271,11 +271,6 @@ struct FastMath {
     return fma(c4, d4, fma(c3, d3, fma(c2, d2, fma(c1, d1, c0 * d0)))) + q2;
   }
 
-  // the restricted stencil with theta = 0, from its cell values
-  __device__ __forceinline__ static double central6(const double* q) {
-    return linear_theta(q[1] - q[0], q[2] - q[1], q[3] - q[2], q[4] - q[3], q[5] - q[4], q[2], false);
-  }
-
   // |x| as the high word of its bit pattern (orders like |x| for finite x; inf and NaN top it)
   __device__ __forceinline__ static int hw(double x) { return __double2hiint(x) & 0x7fffffff; }
   // The high 32 bits of a double as a float: its sign, its exponent rebiased and the top 20
