@@ -57,10 +57,10 @@ struct Tile1D {
   static_assert(!DP || M == 3, "differences first: 1D Euler tiles");
   static constexpr int kRed = kDu + (DP ? (LATE ? 1 : 2) * M * W : 0);
   static constexpr int kQn = kRed + 4 * 32;      // queue length (int)
-  // queue of reconstructions still to be completed: one slot per thread, fewer if the tile
-  // would pass 48 KB (the rest are completed in place).  A record holds the weights' inputs
-  // (9 doubles), or with SPLIT = 2 a stencil's differences (15 doubles, FastMath::kDeferRec)
-  static constexpr int REC = (SPLIT == 2) ? 15 : 9;
+  // queue of reconstructions still to be completed (DP; the screened scalar tiles list their
+  // interfaces here): one slot per thread, fewer if the tile would pass 48 KB (the rest are
+  // completed in place).  A record holds the weights' inputs
+  static constexpr int REC = 9;
   static constexpr int kQ = kQn + 2;             // queue records [REC][QCAP]
   static constexpr int kQFit = ((48 * 1024 / 8 - kQ) * 2) / (2 * REC + 1);
   static constexpr int QCAP = (kQFit < NT ? kQFit : NT) & ~1;
@@ -1131,22 +1131,8 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
     }
   };
 
-  // ---- C0: Roe average and left eigenvectors per interface (interface i: cells i+2 | i+3);
-  // with MATH::kRoeRows one row of the matrix per thread
-  if (FLUX == WT_FLUX_EULER1D && MATH::kRoeRows) {
-    if (tid < 3 * ni) {
-      const int row = tid / ni, i = tid - row * ni;
-      double l[3], rs[3];
-      MATH::roe_row(s_sr[i + 2], s_vel[i + 2], s_H[i + 2], s_sr[i + 3], s_vel[i + 3], s_H[i + 3], a.gamma, row, l, rs);
-#pragma unroll
-      for (int e = 0; e < 3; ++e) s_L[(3 * row + e) * NI + i] = l[e];
-      if (row == 0) {
-#pragma unroll
-        for (int e = 0; e < 3; ++e) s_rs[e * NI + i] = rs[e];
-      }
-    }
-    c0_barrier();
-  } else if (FLUX == WT_FLUX_EULER1D) {
+  // ---- C0: Roe average and left eigenvectors per interface (interface i: cells i+2 | i+3)
+  if (FLUX == WT_FLUX_EULER1D) {
     for (int i = tid; i < ni; i += NT) {
       double L[9], rs[3];
       MATH::roe(s_sr[i + 2], s_vel[i + 2], s_H[i + 2], s_sr[i + 3], s_vel[i + 3], s_H[i + 3], a.gamma, L, rs);
@@ -1270,46 +1256,9 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   // records are written (phase E reuses it afterwards)
   unsigned char* s_fl = reinterpret_cast<unsigned char*>(s_red);
   static_assert(!REC || (2 * M * NI <= 4 * 32 * 8 && MODE == kStage), "flags fit the reduction buffer");
-  // one reconstruction (stencil q) into s_F[dst], or into the queue
+  // one reconstruction (stencil q) into s_F[dst]
   auto reconstruct = [&](const double* q, const int dst) {
-    if constexpr (MATH::kSplitWeno && MODE == kStepBlocked) {
-      // a stencil the FP32 screen does not settle is deferred whole to the quad pass, so the
-      // long FP64 path never diverges inside the warps of this pass
-      double rec[TL::REC];
-      double out;
-      if (MATH::weno_front(q, a.eps, a.alpha_R, out, rec)) {
-        s_F[dst] = out;
-      } else {
-        const int slot = atomicAdd(s_qn, 1);
-        if (slot < QCAP) {
-#pragma unroll
-          for (int r = 0; r < TL::REC; ++r) s_q[r * QCAP + slot] = rec[r];
-          s_qi[slot] = dst;
-        } else {
-          s_F[dst] = MATH::weno(q, a.eps, a.alpha_R);
-        }
-      }
-    } else if constexpr (MATH::kSplitWeno) {
-      typename MATH::WenoPart w;
-      double out;
-      if (MATH::weno_begin(q, a.eps, a.alpha_R, out, w)) {
-        s_F[dst] = out;
-        if constexpr (REC) s_fl[dst] = (unsigned char)(1 | (w.theta1 ? 2 : 0));
-      } else {
-        if constexpr (REC) s_fl[dst] = (unsigned char)(w.theta1 ? 2 : 0);
-        const int slot = atomicAdd(s_qn, 1);
-        if (slot < QCAP) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) s_q[k * QCAP + slot] = w.e[k];
-          s_q[4 * QCAP + slot] = w.tau;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) s_q[(5 + k) * QCAP + slot] = w.fh[k];
-          s_qi[slot] = dst | (w.theta1 ? (1 << 30) : 0);
-        } else {
-          s_F[dst] = MATH::weno_finish(w);
-        }
-      }
-    } else if constexpr (REC) {
+    if constexpr (REC) {
       bool r, t;
       s_F[dst] = MATH::weno_flags(q, a.eps, a.alpha_R, r, t);
       s_fl[dst] = (unsigned char)((r ? 1 : 0) | (t ? 2 : 0));
@@ -1420,27 +1369,9 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
       for (int c = 0; c < M; ++c) bulk_g2s(s_un + c * W, a.un + c * a.pitch + s0, late_bytes, s_bar);
     }
   }
-  if constexpr (MATH::kSplitWeno) {
+  if constexpr (DP) {
     const int nq = min(*s_qn, QCAP);  // the same for every thread of the block
-    if (nq > 0 && MODE == kStepBlocked) {
-      // a quad of lanes per deferred stencil (FastMath::weno_back_quad): lane k forms
-      // indicator k and weight k, the quad shares them by shuffles, and its lane 0 holds the
-      // result.  The tiles holding a shock carry the queue, and every CTA waits for them at
-      // the next alpha exchange.
-      for (int base = 0; base < nq; base += NT / 4) {
-        const int t = base + (tid >> 2), k = tid & 3;
-        if (t < nq) {  // the same for the four lanes of a quad
-          double rec[TL::REC];
-#pragma unroll
-          for (int r = 0; r < TL::REC; ++r) rec[r] = s_q[r * QCAP + t];
-          const unsigned qmask = 0xfu << (tid & 28);
-          const double out = MATH::weno_back_quad(k, rec, a.eps, a.alpha_R, qmask);
-          const int qi = s_qi[t];  // bit 30: a negated - side stencil
-          if (k == 0) s_F[qi & ((1 << 30) - 1)] = flip_sign(out, (qi >> 30) & 1 ? 0x8000000000000000ull : 0ull);
-        }
-      }
-      __syncthreads();
-    } else if (nq > 0) {
+    if (nq > 0) {
       for (int t = tid; t < nq; t += NT) {
         typename MATH::WenoPart w;
 #pragma unroll

@@ -19,7 +19,6 @@ namespace wt {
 
 struct FastMath {
   static constexpr bool kStrict = false;
-  static constexpr bool kRoeRows = false;  // Roe matrix one row per thread (roe_row)
   // projection v = kProj (L f +- alpha L u) with the stored L = kLScale * L_true
   static constexpr double kProj = 1.0, kLScale = 0.5;
 
@@ -157,34 +156,6 @@ struct FastMath {
     rs[2] = c;
   }
 
-  // Roe's mean state and row `row` of the (1/2-scaled) left eigenvectors, the rows written as
-  // one formula with row-dependent coefficients (no divergence between rows); rs as in roe
-  __device__ __forceinline__ static void roe_row(double sa, double ua, double Ha, double sb, double ub, double Hb,
-                                                 double gamma, int row, double* l, double* rs) {
-    const double is = 1.0 / (sa + sb);
-    const double wa = sa * is, wb = sb * is;
-    const double u = dot2(wa, ua, wb, ub);
-    const double H = dot2(wa, Ha, wb, Hb);
-    const double gm1 = gamma - 1.0;
-    const double c2 = gm1 * fma(-0.5 * u, u, H);
-    const double ic = rsqrt(c2);
-    const double hb1 = 0.5 * gm1 * ic * ic;
-    const double hb2 = 0.5 * u * u * hb1;
-    const double uic = 0.5 * u * ic;
-    const double hb1u = hb1 * u;
-    // rows: (0.5 (hb2 + uic), -0.5 hb1u - 0.25 ic, 0.5 hb1), (0.5 - hb2, hb1u, -hb1),
-    //       (0.5 (hb2 - uic), -0.5 hb1u + 0.25 ic, 0.5 hb1)
-    const double A = row == 1 ? -1.0 : 0.5, B = row == 0 ? 0.5 : (row == 1 ? 0.0 : -0.5);
-    const double C = row == 1 ? 0.5 : 0.0, D = row == 1 ? 1.0 : -0.5;
-    const double E = row == 0 ? -0.25 : (row == 1 ? 0.0 : 0.25), F = row == 1 ? -1.0 : 0.5;
-    l[0] = fma(A, hb2, fma(B, uic, C));
-    l[1] = fma(D, hb1u, E * ic);
-    l[2] = F * hb1;
-    rs[0] = u;
-    rs[1] = H;
-    rs[2] = c2 * ic;
-  }
-
   __device__ __forceinline__ static void project3(const double* l, const double* f, const double* U, double alpha,
                                                   double& vp, double& vm) {
     const double a = fma(l[2], f[2], fma(l[1], f[1], l[0] * f[0]));
@@ -243,7 +214,6 @@ struct FastMath {
   // indicators, tau and the theta switch; a restricted stencil (Eq. (be_res)) finishes there
   // with the linear combination (returns true, value in out).  Otherwise the nonlinear
   // weights of Eq. (om) are left to weno_finish, which needs only the record w.
-  static constexpr bool kSplitWeno = true;
   struct WenoPart {
     double e[4];   // eps + beta_k
     double tau;    // tau^theta
@@ -387,22 +357,13 @@ struct FastMath {
     return false;
   }
 
-  // ---- The reconstruction in a front and a back half, for the step-blocked kernel.
-  // weno_front takes the differences, the large-stencil terms and the FP32 screen; a screened
-  // stencil finishes there (linear scheme, returns true).  Any other stencil leaves a record of
-  // kDeferRec doubles (d0..d4, s0..s3, t5a, t5b, t6a, t6b, q2, q3) that a quad of lanes
-  // completes in weno_back_quad with the operations of weno_begin's FP64 path and of
-  // weno_finish, so the value is the same as theirs.
-  static constexpr int kDeferRec = 15;
-  __device__ __forceinline__ static bool weno_front(const double* q, double eps, double alpha_R, double& out,
-                                                    double* rec) {
-    const double d0 = q[1] - q[0], d1 = q[2] - q[1], d2 = q[3] - q[2], d3 = q[4] - q[3], d4 = q[5] - q[4];
-    const int scr = weno_front_core<false>(d0, d1, d2, d3, d4, q[2], q[3], eps, alpha_R, rec);
-    if (scr != 0) out = linear_theta(d0, d1, d2, d3, d4, q[2], scr == 1);
-    return scr != 0;
-  }
-  // the same from the stencil's differences and q_2 (q_3 taken as q_2 + d_2), the linear scheme left
-  // to the caller: returns the screen's verdict, 1 (theta = 1), 2 (theta = 0) or 0 (a record)
+  // ---- The reconstruction in a front and a back half, for the latency-bound tiles.  weno_front_d
+  // takes the stencil's differences and q_2 (q_3 taken as q_2 + d_2): the large-stencil terms and
+  // the FP32 screen.  The linear scheme of a screened stencil is left to the caller: returns the
+  // screen's verdict, 1 (theta = 1), 2 (theta = 0) or 0.  With 0 it leaves a record of 15 doubles
+  // (d0..d4, s0..s3, t5a, t5b, t6a, t6b, q2, q3) that a quad of lanes completes in
+  // weno_back_quad with the operations of weno_begin's FP64 path and of weno_finish, so the
+  // value is the same as theirs.
   __device__ __forceinline__ static int weno_front_d(const double* d, double q2, double eps, double alpha_R,
                                                      double* rec) {
     return weno_front_core<true>(d[0], d[1], d[2], d[3], d[4], q2, 0.0, eps, alpha_R, rec);

@@ -11,20 +11,10 @@ namespace wt {
 struct StrictMath {
   static constexpr bool kStrict = true;
   static constexpr bool kCentral = false;  // no central screen (wt_central.cuh): every reconstruction is evaluated
-  static constexpr bool kRoeRows = false;  // the whole Roe matrix per interface (roe)
   // projection v = kProj (L f +- alpha L u) with the stored L = kLScale * L_true
   static constexpr double kProj = 0.5, kLScale = 1.0;
-  // the reconstruction is evaluated in one piece (weno_flags)
-  static constexpr bool kSplitWeno = false;
   // the projections are taken cell by cell, in the order of Eq. (flux_split_lf)
   static constexpr bool kDiffProj = false;
-  struct WenoPart {
-    double e[4], tau, fh[4];
-    bool theta1;
-  };
-  __device__ __forceinline__ static bool weno_begin(const double*, double, double, double&, WenoPart&) { return true; }
-  __device__ __forceinline__ static double weno_finish(const WenoPart&) { return 0.0; }
-
   // ---- scalar fluxes (Eq. (lin_eq), Eq. (bur_eq))
   __device__ __forceinline__ static double flux_advection(double a, double u) { return a * u; }
   __device__ __forceinline__ static double flux_burgers(double u) { return 0.5 * u * u; }
@@ -104,9 +94,6 @@ struct StrictMath {
     rs[1] = H;
     rs[2] = c;
   }
-
-  __device__ __forceinline__ static void roe_row(double, double, double, double, double, double, double, int,
-                                                 double*, double*) {}
 
   // ---- Global Lax-Friedrichs splitting of one projected cell (Eq. (flux_split_lf))
   __device__ __forceinline__ static void project3(const double* l, const double* f, const double* U, double alpha,
