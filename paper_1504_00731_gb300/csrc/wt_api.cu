@@ -889,7 +889,12 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   double* U2 = reinterpret_cast<double*>(w + lay.u2);
   double* st_in = reinterpret_cast<double*>(w + lay.st_in);
   const double dx = (grid->hi[0] - grid->lo[0]) / (double)n;
-  const int tile = default_tile(prob->flux, n);
+  // Fast Euler: the 63-cell tile spreads a shock's FP64 path over 192 threads, the 127-cell one runs
+  // it on 64, so four to eight 63-cell tiles per SM are the faster on grids with a shock and as fast
+  // on smooth ones (60 steps of Riemann data on 40011, 55011, 70011 cells: 8.9, 9.4, 10.1 ms with
+  // 127, 4.6, 5.0, 5.5 with 63; smooth data on 45011: 4.2 both)
+  const bool mid = prob->flux == WT_FLUX_EULER1D && prob->mode != WT_MODE_STRICT && n > 152LL * 31 && n <= 152LL * 8 * 63;
+  const int tile = mid ? 63 : default_tile(prob->flux, n);
 
   const Ctl h = make_ctl(cfl, dt_fixed, t_final);
   WT_CUDA(cudaMemcpyAsync(ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
