@@ -937,7 +937,7 @@ __device__ __forceinline__ bool scalar_fluxes(const Stage1DArgs& a, const int Tc
         MATH::project1_ab(s_f[c], s_u[c], x, y);
         q[z] = MATH::project_side(x, y, alpha[0], side != 0);
       }
-      F = MATH::weno(q, a.eps, a.alpha_R);
+      F = MATH::weno_scalar(q, a.eps, a.alpha_R);
     }
     const double o = __shfl_xor_sync(0xffffffffu, F, 1);
     if (has && side == 0) s_h[i] = F + o;

@@ -483,6 +483,24 @@ struct FastMath {
     bool r, t;
     return weno_flags(q, eps, alpha_R, r, t);
   }
+  // weno for the scalar fluxes.  The common denominator prod_l (eps + beta_l) of weno_finish overflows from about
+  // beta = 2^220 on, which Burgers data of 2^55 reach (f = u^2 / 2).  The weights of Eq. (om) do not
+  // change if every eps + beta_l and tau are scaled alike: by the power of two that brings the largest
+  // to 2^128, where it is at 2^200 or above.  (Not in weno_finish itself: the branch in the Euler
+  // tiles' weights cost 1.5 to 2 % of runs with shocks, and Euler data reach it from 2^100 on only.)
+  __device__ __forceinline__ static double weno_scalar(const double* q, double eps, double alpha_R) {
+    WenoPart w;
+    double out;
+    if (weno_begin(q, eps, alpha_R, out, w)) return out;
+    const int h = max(max(hw(w.e[0]), hw(w.e[1])), max(hw(w.e[2]), hw(w.e[3])));
+    if (h >= ((1023 + 200) << 20)) {
+      const double sc = __hiloint2double((int)(((2046u + 128u) << 20) - ((unsigned)h & 0x7ff00000u)), 0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w.e[k] *= sc;
+      w.tau *= sc;
+    }
+    return weno_finish(w);
+  }
   __device__ __forceinline__ static double weno_d(const double* d, double q2, double eps, double alpha_R) {
     WenoPart w;
     double out;
