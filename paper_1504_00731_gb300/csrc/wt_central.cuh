@@ -65,6 +65,18 @@ __device__ __forceinline__ float2 f32_pair(double x) {
   return make_float2(__int_as_float(t | sg), __int_as_float(__float_as_int(tail) ^ sg));
 }
 
+// the same with a nonzero high part for every x other than zero
+__device__ __forceinline__ float2 f32_pair_nz(double x) {
+  float2 p = f32_pair(x);
+  const unsigned any = ((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x);
+  if (p.x == 0.0f && any != 0u) p.x = 0x1p-126f;
+  return p;
+}
+
+// whether eps and alpha_R (as floats) are in the screen's range: the thresholds of Eq. (be_res) are then
+// normal floats
+__device__ __forceinline__ bool screen_constants(float eps, float aR) { return fmul(aR, eps) > 1e-30f && eps > 0x1p-120f; }
+
 // a - b of FP32 pairs: the high parts' difference and its exact rounding error, plus the low
 // parts' (not renormalised; the low part's own roundings stay below 2^-46 of the largest input)
 __device__ __forceinline__ float2 pair_sub(float2 a, float2 b) {

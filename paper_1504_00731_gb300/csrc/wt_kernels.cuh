@@ -534,7 +534,7 @@ __device__ __forceinline__ bool central_fluxes_blocked(const Stage1DArgs& a, con
     named_barrier_sync(4, NP + 32);  // the speed warp holds the alphas of every CTA
 #pragma unroll
     for (int f = 0; f < 3; ++f) alpha[f] = bits_to_double(s_alpha[f]);
-    if (has && !(fmul(aR, eps) > 1e-30f && z.prove(s, alpha, eps, aR))) atomicOr(&s_mark[i], 1 << s);
+    if (has && !(screen_constants(eps, aR) && z.prove(s, alpha, eps, aR))) atomicOr(&s_mark[i], 1 << s);
   } else if ((tid >> 5) != kSW) {
     if (tid - NP < ni) central_roe<MATH, TL>(a, sm, off, tid - NP, tid - NP);
   } else {
@@ -629,7 +629,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
 
   // ---- D2
   const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
-  const bool screenable = fmul(aR, eps) > 1e-30f;
+  const bool screenable = screen_constants(eps, aR);
   auto central = [&](const int c, const int i) { s_h[c * NI + i] = central_flux<TL>(sm, c, i); };
   if constexpr (kThree) {
     const bool has = tid < 3 * ni;
@@ -822,8 +822,8 @@ __device__ __forceinline__ bool scalar_fluxes(const Stage1DArgs& a, const int Tc
     for (int k = tid; k < nd; k += NP) {
       const double df = __dsub_rn(s_f[k + 1], s_f[k]);
       s_df[k] = df;
-      s_pair[k] = f32_pair(df);
-      s_pair[W + k] = f32_pair(__dsub_rn(s_u[k + 1], s_u[k]));
+      s_pair[k] = f32_pair_nz(df);
+      s_pair[W + k] = f32_pair_nz(__dsub_rn(s_u[k + 1], s_u[k]));
     }
   }
   if (MODE != kStepBlocked) {
@@ -898,7 +898,14 @@ __device__ __forceinline__ bool scalar_fluxes(const Stage1DArgs& a, const int Tc
       } else {
         verdict = prove_field(fa[e], fb[e], ea, eb, al, fmul(4.0f, eps), aR, fmul(60.0f * 0x1p-53f, gm));
       }
-      if (!(big < 0x1p60f && fmul(aR, eps) > 1e-30f)) verdict = 0;
+      // The pairs lose what lies below 2^-126: 2^-121 in a fifth difference.  That is within the pairs' own
+      // error above (2^-41 of the largest, taken as 2^-40) from 2^-78 on, for f as for alpha u
+      // (advection: f alone); all differences zero (exactly: f32_pair_nz) is decided whatever their size.
+      constexpr float kLow = 0x1p-78f;
+      const bool enough = FLUX == WT_FLUX_ADVECTION ? am[e] >= kLow || am[e] == 0.0f
+                                                    : (bm[e] >= kLow && fmaxf(am[e], fmul(al, bm[e])) >= kLow) ||
+                                                          (am[e] == 0.0f && bm[e] == 0.0f);
+      if (!(big < 0x1p60f && enough && screen_constants(eps, aR))) verdict = 0;
       if (verdict == 0) {
         s_list[atomicAdd(&s_cnt[2], 1)] = i;
       } else {

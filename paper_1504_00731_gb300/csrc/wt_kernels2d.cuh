@@ -146,7 +146,7 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
   __syncthreads();
   // ---- D2
   const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
-  const bool screenable = fmul(aR, eps) > 1e-30f;
+  const bool screenable = screen_constants(eps, aR);
   for (int it = tid; it < ni; it += NT) {
     const int r = it / nper, i = it - r * nper;
     const int k0 = DIR == 0 ? (r + G) * WX + i : r * WX + i + G;  // first stencil cell
