@@ -336,11 +336,12 @@ __global__ void __launch_bounds__(KernelTile2D<MATH, TX, TY>::NT, KernelTile2D<M
   const int tid = threadIdx.x;
   Ctl* ctl = a.ctl;
   const long long nx = a.nx, ny = a.ny;
-  const long long x0 = (long long)blockIdx.x * TX, y0 = (long long)blockIdx.y * TY;
+  // (a grid dimension holds 65535 rows of tiles; the rest are on z)
+  const long long x0 = (long long)blockIdx.x * TX, y0 = (blockIdx.y + (long long)blockIdx.z * gridDim.y) * TY;
   if (x0 >= nx || y0 >= ny) return;
   const int tcx = (int)((nx - x0 < TX) ? (nx - x0) : TX);
   const int tcy = (int)((ny - y0 < TY) ? (ny - y0) : TY);
-  const bool first_tile = (blockIdx.x == 0 && blockIdx.y == 0);
+  const bool first_tile = x0 == 0 && y0 == 0;
 
   double dt = 0.0;
   if (STAGE != STAGE_RHS) {
@@ -713,7 +714,8 @@ cudaError_t launch_stage2d_t(const Stage2DArgs& a, cudaStream_t st) {
   constexpr int TY = kTileY<MATH>;
   using TL = KernelTile2D<MATH, TX, TY>;
   auto kern = stage2d_kernel<MATH, STAGE, TX, TY>;  // prepare_stage2d_policy() raised its shared-memory limit
-  dim3 grid((unsigned)((a.nx + TX - 1) / TX), (unsigned)((a.ny + TY - 1) / TY));
+  const long long rows = (a.ny + TY - 1) / TY, ny = rows < 65535 ? rows : 65535;
+  dim3 grid((unsigned)((a.nx + TX - 1) / TX), (unsigned)ny, (unsigned)((rows + ny - 1) / ny));
   return launch_pdl(kern, grid, dim3(TL::NT), TL::bytes, st, a);
 }
 
