@@ -161,6 +161,12 @@ __device__ __forceinline__ float field_err(int s, const Roe32& r, float2 nb, flo
                 : ffma(r.rel, fadd(aj, ak), fmul(r.q, fadd(nb.x, nb.y)));
 }
 
+// The least value of the largest cell difference of a component in the error bounds.  The pairs lose what
+// lies below 2^-125, 2^-121 in a fifth difference, whatever the differences' own size: with this
+// floor the pairs' error 2^-40 max |d| covers it too.  (Cold or thin gas, rho c^3 below 2^-74:
+// there the loss is above 60 * 2^-53 rho c after the product with b1 = (gamma - 1) / c^2.)
+constexpr float kLow32 = 0x1p-80f;
+
 // The projections of one array (f or u) over an interface's stencil, before the field is chosen:
 // d[c] the high parts of component c's five differences, h[c] its high differences.  [0..4]
 // the cell differences, [5..8] third, fourth, fourth, fifth.
@@ -171,8 +177,9 @@ struct Proj32 {
   float jm, km, xm;  // max |j|, |k|, |x0| over the cell differences
 };
 __device__ __forceinline__ void project_stencil(const Roe32& r, const float (*d)[5], const float4* h, Proj32& p) {
-  p.jm = p.km = p.xm = 0.0f;
-  float m1 = 0.0f, m2 = 0.0f;
+  p.jm = p.km = 0.0f;
+  p.xm = kLow32;
+  float m1 = kLow32, m2 = kLow32;
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     p.jk[k] = project32(r, d[0][k], d[1][k], d[2][k]);
@@ -342,7 +349,7 @@ __device__ __forceinline__ void project_stencil_2d(const Roe32Shear& o, const fl
                                                    Proj32Shear& p) {
   const Roe32& r = o.r;
   p.jm = p.km = p.xm = p.tm = 0.0f;
-  float mx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  float mx[4] = {kLow32, kLow32, kLow32, kLow32};
 #pragma unroll
   for (int v = 0; v < 9; ++v) {
     float x[4];
