@@ -275,7 +275,8 @@ __device__ __forceinline__ int prove_field(const float* a, const float* b, const
       const float hi3 = fadd(t3, ehi[0]), hi4 = fadd(fabsf(ty), ehi[y - 5]);
       const float lo5 = fmaxf(fsub(a5, ehi[3]), 0.0f), lo6 = fmaxf(fsub(a6, e6), 0.0f);
       const float tau5hi = ffma(fmul(F1312, hi4), hi4, fmul(hi3, hi3));
-      const float tau6lo = ffma(fmul(F1312, lo5), lo5, fmul(0.25f, fmul(lo6, lo6)));
+      // (halved before the square: a bound that overflows must be one whose value does)
+      const float hl6 = fmul(0.5f, lo6), tau6lo = ffma(fmul(F1312, lo5), lo5, fmul(hl6, hl6));
       ok = ok && fmul(tau5hi, 1.0f + 0x1p-18f) < tau6lo && tau6lo > 0x1p-100f;
       verdict |= side ? 4 : 2;
     }

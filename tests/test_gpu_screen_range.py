@@ -1,6 +1,6 @@
 """The fast Euler screens (wt_central.cuh) at the ends of FP32's range: gas so cold or thin that the products
 with 1 / c^2 raise what the FP32 pairs lose below 2^-125 above the threshold under which theta does not
-matter."""
+matter, and data whose indicators' squares pass 2^128."""
 import numpy as np
 import pytest
 
@@ -38,3 +38,18 @@ def test_rhs_of_cold_and_thin_gas(wtlib, oracle, shape, a, c, amp):
         _check(wtlib, oracle, wtlib.WT_FLUX_EULER1D, W.cons_1d(r, one, p), (1.0 / shape[0],))
     else:
         _check(wtlib, oracle, wtlib.WT_FLUX_EULER2D, W.cons_2d(r, one, 0.5 * one, p), (1.0 / shape[1], 1.0 / shape[0]))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", [-2, -1, 0, 1, 2])
+def test_rhs_2d_of_dense_fast_streams(wtlib, oracle, k):
+    """Noise of 2^k in the transverse velocity of a stream with rho u = 2^60 beside one twice as fast (so that
+    neither side of the splitting vanishes): the squares of the fourth differences' sums lie on
+    both sides of 2^128.  The same bounds."""
+    rng = np.random.default_rng(12)
+    ny, nx = shape = (24, 600)
+    u = np.where(np.arange(nx) < nx - 8, 2.0**10, 2.0**11) * np.ones(shape)
+    U = W.cons_2d(np.full(shape, 2.0**50), u, 2.0**k * rng.uniform(-1, 1, shape), np.full(shape, 2.0**70))
+    _check(wtlib, oracle, wtlib.WT_FLUX_EULER2D, U, (1.0 / nx, 1.0 / ny))
+    V = np.ascontiguousarray(U[[0, 2, 1, 3]].transpose(0, 2, 1))
+    _check(wtlib, oracle, wtlib.WT_FLUX_EULER2D, V, (1.0 / ny, 1.0 / nx))
