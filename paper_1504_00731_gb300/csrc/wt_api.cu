@@ -894,7 +894,7 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   // on smooth ones (60 steps of Riemann data on 40011, 55011, 70011 cells: 8.9, 9.4, 10.1 ms with
   // 127, 4.6, 5.0, 5.5 with 63; smooth data on 45011: 4.2 both)
   const bool mid = prob->flux == WT_FLUX_EULER1D && prob->mode != WT_MODE_STRICT && n > 152LL * 31 && n <= 152LL * 8 * 63;
-  const int tile = mid ? 63 : default_tile(prob->flux, n);
+  int tile = mid ? 63 : default_tile(prob->flux, n);
 
   const Ctl h = make_ctl(cfl, dt_fixed, t_final);
   WT_CUDA(cudaMemcpyAsync(ctl, &h, sizeof(Ctl), cudaMemcpyHostToDevice, st));
@@ -923,7 +923,7 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   WT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int tsb = stepblock1d_tile(prob->flux, n, nsm);
   const long long nsb = (n + tsb - 1) / tsb;
-  const long long ntiles = (n + tile - 1) / tile;
+  long long ntiles = (n + tile - 1) / tile;
   int kind = 0, pgrid = 0;
   if (max_steps > 0 && prob->launch == WT_LAUNCH_AUTO) {
     const int cap_sb = strict ? stepblock1d_capacity_strict(prob->flux, tsb) : stepblock1d_capacity_fast(prob->flux, tsb);
@@ -931,6 +931,15 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
       kind = 2;
       pgrid = (int)nsb;
     } else {
+      // Fast Euler: 31-cell tiles as long as they are co-resident.  A stage lasts as long as the tile with a
+      // front, whose FP64 path is half as long there (us per stage with 63 and with 31 cells:
+      // 9,001 cells of Riemann data 19.4, 16.5, blast waves 25.1, 19.6, smooth 7.7, 7.7; 14,001 cells
+      // 19.0, 17.1; 24.0, 20.5; 10.2, 10.2)
+      if (tile == 63 && prob->flux == WT_FLUX_EULER1D && !strict &&
+          (n + 30) / 31 <= persist1d_capacity_fast(prob->flux, 31)) {
+        tile = 31;
+        ntiles = (n + 30) / 31;
+      }
       const int cap = strict ? persist1d_capacity_strict(prob->flux, tile) : persist1d_capacity_fast(prob->flux, tile);
       if (cap > 0 && ntiles <= cap) {
         kind = 1;

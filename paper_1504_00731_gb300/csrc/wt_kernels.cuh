@@ -80,8 +80,14 @@ struct TileC {
   static constexpr int M = 3;
   static constexpr int W = (T + 9) & ~1;
   static constexpr int NI = T + 1;
-  static constexpr int NT = NT_;
   static constexpr bool kThree = IPT == 1;  // three threads per interface (latency-bound tiles)
+  // A warp for the FP64 Roe averages of every interface while the others screen (central_fluxes): 16 problems of
+  // 64 to 512 cells, 6 steps, 472 -> 421 us; 6,001 cells of Riemann data 17.9 -> 16.6 us per stage (before
+  // the central screen, 16.4)
+  static constexpr bool kRoeWarp = kThree && T == 31 && MODE != kStepBlocked;
+  static constexpr bool kRoeMemory = kRoeWarp && MODE == kResident;  // ... if the tile needed them in the last stage
+  static constexpr int NP = NT_;  // threads of the screen and of the FP64 path
+  static constexpr int NT = NT_ + (kRoeWarp ? 32 : 0);
   static constexpr int FC = kThree ? (NI < 64 ? NI : 64) : (NI < 32 ? NI : 32);
   static constexpr int kBar = 0;
   static constexpr int kUin = 2;
@@ -92,21 +98,23 @@ struct TileC {
   static constexpr int kSr = kH + W;        // sqrt(rho): step-blocked tiles only
   static constexpr int kD = kSr + (MODE == kStepBlocked ? W : 0);  // [6][W] f_{k+1} - f_k, then u_{k+1} - u_k
   static constexpr int kPair = kD + 6 * W;  // [6][W] the differences as FP32 pairs
-  // FP64 path: [9][FC], then [3][FC], [6][FC], over the pairs; after them in the step-blocked tiles,
-  // whose Roe averages are taken while the screen runs
-  static constexpr int kL = kPair + (MODE == kStepBlocked ? 6 * W : 0);
-  static constexpr int kPairN = (MODE == kStepBlocked || 18 * FC > 6 * W) ? kL - kPair + 18 * FC : 6 * W;
+  // FP64 path: [9][FC], then [3][FC], [6][FC], over the pairs; after them in the tiles whose Roe averages
+  // are taken while the screen runs
+  static constexpr bool kRoeAhead = MODE == kStepBlocked || kRoeWarp;
+  static constexpr int kL = kPair + (kRoeAhead ? 6 * W : 0);
+  static constexpr int kPairN = (kRoeAhead || 18 * FC > 6 * W) ? kL - kPair + 18 * FC : 6 * W;
   static constexpr int kRs = kL + 9 * FC;
   static constexpr int kFs = kRs + 3 * FC;
   static constexpr int kHf = kPair + kPairN + (kPairN & 1);  // [3][NI] interface fluxes
   static constexpr int kRed = kHf + 3 * NI;
-  static constexpr int kQn = kRed + 4 * 32;     // ints: queue length, flag of the kernel, listed interfaces
+  static constexpr int kQn = kRed + 4 * 32;     // ints: queue length, flag of the kernel, listed interfaces, of the stage before
   static constexpr int kList = kQn + 2;         // ints [NI]: interfaces of the FP64 path; ints [NI]: marks
   static constexpr int kQ = (kList + NI + 1) & ~1;
   // queue of the FP64 path's unfinished reconstructions; before it, the high differences of a
   // screen spread over three threads per interface (float4 [6][NI])
   static constexpr int REC = kThree ? 15 : 9;
-  static constexpr int QCAP = kThree ? 96 : 64;
+  // (resident tiles: half of all stencils of 63 cells, all of 31; blast waves overflow 96 records)
+  static constexpr int QCAP = kThree ? (MODE == kResident ? (6 * FC < 192 ? 6 * FC : 192) : 96) : 64;
   static constexpr int kQi = kQ + REC * QCAP;
   static constexpr int kQN = REC * QCAP + QCAP / 2;
   static constexpr int kTotal = kQ + (kThree && 12 * NI > kQN ? 12 * NI : kQN);
@@ -373,10 +381,13 @@ __device__ __forceinline__ double central_flux(const double* sm, int c, int i) {
   const double* f = sm + TL::kF + c * TL::W + i;
   return central_value(f[2], f[3], d[0], d[1], d[3], d[4]);
 }
-// FP64 path: Roe average and eigenvectors of interface i into slot q
-template <class MATH, class TL>
+// FP64 path: Roe average and eigenvectors of interface i into slot q.  AHEAD: on the Roe warp, which arrives at
+// barrier 4 once the inputs are read.
+template <class MATH, class TL, bool AHEAD = false>
 __device__ __forceinline__ void central_roe(const Stage1DArgs& a, double* sm, int off, int i, int q) {
-  const double *r = sm + TL::kUin + off + i + 2, *v = sm + TL::kVel + i + 2, *H = sm + TL::kH + i + 2;
+  const double *pr = sm + TL::kUin + off + i + 2, *pv = sm + TL::kVel + i + 2, *pH = sm + TL::kH + i + 2;
+  const double r[2] = {pr[0], pr[1]}, v[2] = {pv[0], pv[1]}, H[2] = {pH[0], pH[1]};
+  if constexpr (AHEAD) named_barrier_arrive(4, TL::NT);
   double L[9], rs[3];
   double sa, sb;
   if constexpr (TL::kD != TL::kSr) {  // taken per cell in phase B
@@ -474,21 +485,32 @@ struct SidePair {
     }
   }
 };
-// a quad of lanes per deferred stencil (FastMath::weno_back_quad)
+// the deferred stencils: a quad of lanes each (FastMath::weno_back_quad) where one round of the block holds
+// them, else a thread each (half the FP64 lane instructions; the same value): 28,001 cells of blast waves
+// 25.9 -> 23.4 us per stage with the longer queue
 template <class MATH, class TL>
 __device__ __forceinline__ void central_deferred(const Stage1DArgs& a, double* sm) {
   const int nq = min(*reinterpret_cast<const int*>(sm + TL::kQn), TL::QCAP);
-  for (int b0 = 0; b0 < nq; b0 += TL::NT / 4) {
-    const int t = b0 + ((int)threadIdx.x >> 2), z = threadIdx.x & 3;
-    if (t < nq) {  // the same for the four lanes of a quad
-      double rec[TL::REC];
+  const int* s_qi = reinterpret_cast<const int*>(sm + TL::kQi);
+  auto put = [&](const int qi, const double v) {
+    sm[TL::kFs + (qi & ((1 << 30) - 1))] = flip_sign(v, (qi >> 30) & 1 ? 0x8000000000000000ull : 0ull);
+  };
+  if (4 * nq > TL::NP) {  // the same for every thread
+    for (int t = threadIdx.x; t < nq; t += TL::NP) {
+      double d[5];
 #pragma unroll
-      for (int y = 0; y < TL::REC; ++y) rec[y] = sm[TL::kQ + y * TL::QCAP + t];
-      const double out = MATH::weno_back_quad(z, rec, a.eps, a.alpha_R, 0xfu << (threadIdx.x & 28));
-      const int qi = reinterpret_cast<const int*>(sm + TL::kQi)[t];
-      if (z == 0)
-        sm[TL::kFs + (qi & ((1 << 30) - 1))] = flip_sign(out, (qi >> 30) & 1 ? 0x8000000000000000ull : 0ull);
+      for (int y = 0; y < 5; ++y) d[y] = sm[TL::kQ + y * TL::QCAP + t];
+      put(s_qi[t], MATH::weno_d(d, sm[TL::kQ + 13 * TL::QCAP + t], a.eps, a.alpha_R));
     }
+    return;
+  }
+  const int t = (int)threadIdx.x >> 2, z = threadIdx.x & 3;
+  if (t < nq) {  // the same for the four lanes of a quad
+    double rec[TL::REC];
+#pragma unroll
+    for (int y = 0; y < TL::REC; ++y) rec[y] = sm[TL::kQ + y * TL::QCAP + t];
+    const double out = MATH::weno_back_quad(z, rec, a.eps, a.alpha_R, 0xfu << (threadIdx.x & 28));
+    if (z == 0) put(s_qi[t], out);
   }
 }
 
@@ -587,8 +609,9 @@ __device__ __forceinline__ bool central_fluxes_blocked(const Stage1DArgs& a, con
 // instructions, no redundant ones).  The others (IPT = 1: latency-bound, three threads or more
 // per interface) give each thread one field, and one component of the high differences,
 // exchanged through shared memory.
+// Returns true where the caller has to wait at barrier 3 (all threads but the Roe warp's) before the next stage.
 template <class MATH, class TL>
-__device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int Tc, const int off,
+__device__ __forceinline__ bool central_fluxes(const Stage1DArgs& a, const int Tc, const int off,
                                                const double (&alpha)[3], double* sm) {
   constexpr int W = TL::W, NI = TL::NI, NT = TL::NT, FC = TL::FC, QCAP = TL::QCAP;
   constexpr bool kThree = TL::kThree;
@@ -605,7 +628,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
   double* s_F = sm + TL::kFs;  // [2 sides * 3 fields][FC]
   double* s_q = sm + TL::kQ;
   int* s_qi = reinterpret_cast<int*>(sm + TL::kQi);
-  int* s_cnt = reinterpret_cast<int*>(sm + TL::kQn);  // [0] queue length, [2] listed interfaces
+  int* s_cnt = reinterpret_cast<int*>(sm + TL::kQn);  // [0] queue length, [2] listed interfaces, [3] of the stage before
   int* s_list = reinterpret_cast<int*>(sm + TL::kList);
   int* s_mark = s_list + NI;
   const int tid = threadIdx.x;
@@ -613,19 +636,50 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
   auto take_diff = [&](const int c, const int k) { central_diff<TL>(sm, off, c, k); };
 
   // ---- D1
+  constexpr int NP = TL::NP;
+  const bool ahead = TL::kRoeMemory ? s_cnt[3] != 0 : TL::kRoeWarp;
+  if constexpr (TL::kRoeWarp) {
+    // The Roe warp takes every interface's average at once (a lane past the last one repeats it), beside the
+    // screen: the chain of a tile with listed interfaces is what a stage of a grid with a front
+    // lasts.  Barriers: 2 the screen's threads, 3 the averages are written, 4 their inputs are
+    // read.  Where nothing is listed nobody waits for the averages before the cells' update.  A
+    // resident tile takes them ahead only if it listed something in the stage before.
+    static_assert(NI == 32 && FC == NI, "an interface per lane of the Roe warp");
+    if (tid >= NP) {
+      const int i = min(tid - NP, ni - 1);
+      if (ahead) {
+        central_roe<MATH, TL, true>(a, sm, off, i, i);
+      } else {
+        named_barrier_arrive(4, NT);
+      }
+      named_barrier_arrive(3, NT);
+      return false;
+    }
+  }
+  auto sync = [&]() {
+    if constexpr (TL::kRoeWarp) {
+      named_barrier_sync(2, NP);
+    } else {
+      __syncthreads();
+    }
+  };
   if (kThree) {
-    for (int idx = tid; idx < 6 * W; idx += NT) {
+    for (int idx = tid; idx < 6 * W; idx += NP) {
       const int c = idx / W, k = idx - c * W;
       if (k < nd) take_diff(c, k);
     }
-    for (int i = tid; i < NI; i += NT) s_mark[i] = 0;
+    for (int i = tid; i < NI; i += NP) s_mark[i] = 0;
   } else {
     for (int k = tid; k < nd; k += NT) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) take_diff(c, k);
     }
   }
-  __syncthreads();
+  if constexpr (TL::kRoeWarp) {
+    named_barrier_sync(4, NT);
+  } else {
+    __syncthreads();
+  }
 
   // ---- D2
   const float gm1 = f32_trunc(a.gamma - 1.0), eps = f32_trunc(a.eps), aR = f32_trunc(a.alpha_R);
@@ -635,15 +689,15 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
     const bool has = tid < 3 * ni;
     const int s = has ? tid / ni : 0, i = has ? tid - s * ni : 0;
     if (has) central_high<TL>(sm, s, i);
-    __syncthreads();
+    sync();
     if (has) {
       Screen32 z;
       central_project<TL>(sm, off, s, i, gm1, z);
       if (!(screenable && z.prove(s, alpha, eps, aR))) atomicOr(&s_mark[i], 1 << s);
     }
-    __syncthreads();
+    sync();
     // the list (a warp per 32 interfaces), and C f of the others
-    for (int w = tid >> 5; w * 32 < ni; w += NT / 32) {
+    for (int w = tid >> 5; w * 32 < ni; w += NP / 32) {
       int at = 0;
       for (int v = 0; v < w; ++v) at += __popc(__ballot_sync(0xffffffffu, s_mark[32 * v + (tid & 31)] != 0));
       const int q = 32 * w + (tid & 31);
@@ -652,7 +706,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
       if (m) s_list[at + __popc(b & ((1u << (tid & 31)) - 1u))] = q | (s_mark[q] << 16);
       if ((w + 1) * 32 >= ni && (tid & 31) == 0) s_cnt[2] = at + __popc(b);
     }
-    for (int idx = tid; idx < 3 * NI; idx += NT) {
+    for (int idx = tid; idx < 3 * NI; idx += NP) {
       const int c = idx / NI, q = idx - c * NI;
       if (q < ni && s_mark[q] == 0) central(c, q);
     }
@@ -696,34 +750,43 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
       }
     }
   }
-  __syncthreads();
+  sync();
 
   // ---- D3
   const int nl = s_cnt[2];
+  if (TL::kRoeMemory && tid == 0) s_cnt[3] = nl;
   for (int base = 0; base < nl; base += FC) {
     const int nc = min(nl - base, FC);
-    for (int q = tid; q < nc; q += NT) central_roe<MATH, TL>(a, sm, off, s_list[base + q] & 0xffff, q);
-    __syncthreads();
+    if constexpr (TL::kRoeWarp) {
+      named_barrier_sync(3, NT);  // (one pass: FC = NI)
+    }
+    if (TL::kRoeWarp && !ahead) {
+      for (int q = tid; q < nc; q += NP) central_roe<MATH, TL>(a, sm, off, s_list[q] & 0xffff, s_list[q] & 0xffff);
+      sync();
+    } else if constexpr (!TL::kRoeWarp) {
+      for (int q = tid; q < nc; q += NT) central_roe<MATH, TL>(a, sm, off, s_list[base + q] & 0xffff, q);
+      __syncthreads();
+    }
     auto proj_cell = [&](const double* l, const int k, double& x, double& y) { central_cell<MATH, TL>(sm, off, l, k, x, y); };
     auto proj_diff = [&](const double* l, const int k, double& x, double& y) { central_dcell<MATH, TL>(sm, l, k, x, y); };
     if constexpr (kThree) {
       // two adjacent threads per (interface, field), one per side (SidePair)
-      for (int w0 = (tid >> 5) * 32; w0 < 6 * nc; w0 += NT) {  // warp-uniform
+      for (int w0 = (tid >> 5) * 32; w0 < 6 * nc; w0 += NP) {  // warp-uniform
         const int it = (w0 + (tid & 31)) >> 1;
         const bool has = it < 3 * nc;
         const int s = has ? it / nc : 0, q = it - s * nc;
         SidePair<MATH, TL> p;
-        const int e = has ? s_list[base + q] : 0;
-        p.project(sm, off, has, s, e & 0xffff, q);
-        if (has) p.reconstruct(a, sm, alpha, s, q, !((e >> (16 + s)) & 1));
+        const int e = has ? s_list[base + q] : 0, i = e & 0xffff, slot = TL::kRoeWarp ? i : q;
+        p.project(sm, off, has, s, i, slot);
+        if (has) p.reconstruct(a, sm, alpha, s, slot, !((e >> (16 + s)) & 1));
       }
-      __syncthreads();
+      sync();
       central_deferred<MATH, TL>(a, sm);
-      __syncthreads();
+      sync();
       // one component of h per thread
-      for (int idx = tid; idx < 3 * nc; idx += NT) {
-        const int c = idx / nc, q = idx - c * nc;
-        s_h[c * NI + (s_list[base + q] & 0xffff)] = central_back<MATH, TL>(sm, c, q);
+      for (int idx = tid; idx < 3 * nc; idx += NP) {
+        const int c = idx / nc, q = idx - c * nc, i = s_list[base + q] & 0xffff;
+        s_h[c * NI + i] = central_back<MATH, TL>(sm, c, TL::kRoeWarp ? i : q);
       }
     } else {
       for (int it = tid; it < 3 * nc; it += NT) {
@@ -766,7 +829,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
           }
         }
       }
-      __syncthreads();
+      sync();
       const int nq = min(s_cnt[0], QCAP);
       for (int t = tid; t < nq; t += NT) {
         typename MATH::WenoPart w;
@@ -779,7 +842,7 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
         w.theta1 = (qi >> 30) & 1;
         s_F[qi & ((1 << 30) - 1)] = MATH::weno_finish(w);
       }
-      __syncthreads();
+      sync();
       for (int q = tid; q < nc; q += NT) {
         const int i = s_list[base + q] & 0xffff;
         const double rs[3] = {s_rs[q], s_rs[FC + q], s_rs[2 * FC + q]};
@@ -791,8 +854,9 @@ __device__ __forceinline__ void central_fluxes(const Stage1DArgs& a, const int T
       }
     }
     if (tid == 0) s_cnt[0] = 0;
-    __syncthreads();
+    sync();
   }
+  return TL::kRoeWarp && nl == 0;
 }
 
 // Interface values of a scalar tile (advection, Burgers) by the screen of wt_central.cuh, in place of phase
@@ -1113,6 +1177,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   }
   if (MODE != kStepBlocked) __syncthreads();
   const double* hsrc = s_h;
+  [[maybe_unused]] bool roe_pending = false;
   if constexpr (SCALAR) {
     if (!scalar_fluxes<MATH, FLUX, MODE, TL>(a, Tc, off, alpha, dt, sm, aw)) return false;
     hsrc = s_F;
@@ -1120,7 +1185,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
     if constexpr (MODE == kStepBlocked) {
       if (!central_fluxes_blocked<MATH, TL>(a, Tc, off, alpha, dt, sm, aw)) return false;
     } else {
-      central_fluxes<MATH, TL>(a, Tc, off, alpha, sm);
+      roe_pending = central_fluxes<MATH, TL>(a, Tc, off, alpha, sm);
     }
   } else {
   // step-blocked scalar fluxes have no phase C0: the alphas are awaited here
@@ -1492,7 +1557,17 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   // where the screen does not apply); the FP64 speeds are then taken only for the cells that
   // can hold a maximum of the tile (below)
   constexpr bool kScreen = FLUX == WT_FLUX_EULER1D && MODE == kStage && STAGE != STAGE_RHS;
-  float* s_lam = reinterpret_cast<float*>(CENTRAL ? s_L : s_F);
+  constexpr bool ROE_WARP = [] {
+    if constexpr (CENTRAL) return TL::kRoeWarp;
+    return false;
+  }();
+  // (with a Roe warp, which may still be at work, in the dead buffer of the pairs)
+  float* s_lam;
+  if constexpr (ROE_WARP) {
+    s_lam = reinterpret_cast<float*>(sm + TL::kPair);
+  } else {
+    s_lam = reinterpret_cast<float*>(CENTRAL ? s_L : s_F);
+  }
   float m32[3] = {0.0f, 0.0f, 0.0f};
   const float g32 = f32_hi(a.gamma * (a.gamma - 1.0));
   for (int t = tid; t < Tc; t += NT) {
@@ -1574,6 +1649,9 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
         }
       }
     }
+  }
+  if constexpr (ROE_WARP) {
+    if (roe_pending) named_barrier_sync(3, NT);
   }
   if constexpr (kScreen) {
     // The tile's FP32 maxima m_s.  With e = 2^-14.6 max(m_0, m_2) bounding every cell's error
@@ -1712,7 +1790,7 @@ __device__ __forceinline__ bool stage1d_tile(const Stage1DArgs& a, const long lo
 }
 
 template <class MATH, int FLUX, int STAGE, int T, int IPT>
-__global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) stage1d_kernel(const Stage1DArgs a) {
+__global__ void __launch_bounds__(KernelTile<MATH, FLUX, T, kStage, IPT>::NT) stage1d_kernel(const Stage1DArgs a) {
   using TL = KernelTile<MATH, FLUX, T, kStage, IPT>;
   extern __shared__ __align__(16) double sm[];
   pdl_launch_dependents();
@@ -1726,7 +1804,7 @@ __global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) s
 // Batched stage: a persistent grid walks a table of (problem, tile) work items over many
 // independent problems, each with its own grid, boundary conditions, alphas and dt.
 template <class MATH, int FLUX, int STAGE, int T, int IPT, int USE = kForward>
-__global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m, 1, IPT, true>::NT) stage1d_batched_kernel(const BatchArgs b) {
+__global__ void __launch_bounds__(KernelTile<MATH, FLUX, T, kStage, IPT, USE>::NT) stage1d_batched_kernel(const BatchArgs b) {
   using TL = KernelTile<MATH, FLUX, T, kStage, IPT, USE>;
   extern __shared__ __align__(16) double sm[];
   pdl_launch_dependents();
@@ -1787,7 +1865,7 @@ __device__ __forceinline__ void load_halos(const double* uin, long long pitch, l
 }
 
 template <class MATH, int FLUX, int T>
-__global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m>::NT, 3) persist1d_kernel(const PersistArgs p) {
+__global__ void __launch_bounds__(KernelTile<MATH, FLUX, T, kResident>::NT, 3) persist1d_kernel(const PersistArgs p) {
   constexpr int M = FluxM<FLUX>::m;
   using TL = KernelTile<MATH, FLUX, T, kResident>;
   constexpr int W = TL::W, NT = TL::NT;
@@ -1804,6 +1882,9 @@ __global__ void __launch_bounds__(Tile1D<T, FluxM<FLUX>::m>::NT, 3) persist1d_ke
   unsigned long long nbar = 0;
   const unsigned long long nblk = gridDim.x;
 
+  if constexpr (kCentralTile<MATH, FLUX, kForward>) {
+    if (tid == 0) reinterpret_cast<int*>(sm + TL::kQn)[3] = 1;  // the Roe warp's first stage
+  }
   // window of u^n: stage input and u^n
   for (int idx = tid; idx < M * cells; idx += NT) {
     const int c = idx / cells, k = idx - c * cells;
