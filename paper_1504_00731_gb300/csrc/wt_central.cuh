@@ -350,7 +350,9 @@ __device__ __forceinline__ void project_stencil_2d(const Roe32Shear& o, const fl
                                                    Proj32Shear& p) {
   const Roe32& r = o.r;
   p.jm = p.km = p.xm = p.tm = 0.0f;
-  float mx[4] = {kLow32, kLow32, kLow32, kLow32};
+  // (no floor for tangential momenta that are equal throughout, f32_pair_nz: a sweep along a stream has a
+  // shear field of zeros and a threshold of zero, and takes the central flux)
+  float mx[4] = {kLow32, kLow32, 0.0f, kLow32};
 #pragma unroll
   for (int v = 0; v < 9; ++v) {
     float x[4];
@@ -369,7 +371,10 @@ __device__ __forceinline__ void project_stencil_2d(const Roe32Shear& o, const fl
     }
     if (v >= 4) {  // the bounds of the largest cell difference, then of the high differences
       const int b = v - 4;
-      if (b == 0) p.xm = mx[0];
+      if (b == 0) {
+        p.xm = mx[0];
+        if (mx[2] > 0.0f) mx[2] = fmaxf(mx[2], kLow32);
+      }
       const float y0 = b == 0 ? mx[0] : fabsf(x[0]), y1 = b == 0 ? mx[1] : fabsf(x[1]),
                   y2 = b == 0 ? mx[2] : fabsf(x[2]), y3 = b == 0 ? mx[3] : fabsf(x[3]);
       const float n1 = ffma(r.U, y0, y1), nt = ffma(o.T, y0, y2);

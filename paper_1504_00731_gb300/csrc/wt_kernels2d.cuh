@@ -137,9 +137,10 @@ __device__ __forceinline__ void central_sweep(const Stage2DArgs& a, const int tc
       const double* x = s_fg + comp(c) * NCELL + k;
       const double df = __dsub_rn(x[ST], x[0]);
       s_df[c * ND + p] = df;
-      s_pair[c * ND + p] = f32_pair(df);
+      s_pair[c * ND + p] = c == 2 ? f32_pair_nz(df) : f32_pair(df);
       const double* y = s_uin + comp(c) * NCELL + k;
-      s_pair[(4 + c) * ND + p] = f32_pair(__dsub_rn(y[ST], y[0]));
+      const double dy = __dsub_rn(y[ST], y[0]);
+      s_pair[(4 + c) * ND + p] = c == 2 ? f32_pair_nz(dy) : f32_pair(dy);
     }
   }
   if (tid == 0) s_nl[0] = s_nl[1] = 0;
