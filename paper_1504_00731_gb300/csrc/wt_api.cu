@@ -893,7 +893,9 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   // it on 64, so four to eight 63-cell tiles per SM are the faster on grids with a shock and as fast
   // on smooth ones (60 steps of Riemann data on 40011, 55011, 70011 cells: 8.9, 9.4, 10.1 ms with
   // 127, 4.6, 5.0, 5.5 with 63; smooth data on 45011: 4.2 both)
-  const bool mid = prob->flux == WT_FLUX_EULER1D && prob->mode != WT_MODE_STRICT && n > 152LL * 31 && n <= 152LL * 8 * 63;
+  int nsm = 0;
+  WT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const bool mid = prob->flux == WT_FLUX_EULER1D && prob->mode != WT_MODE_STRICT && n > 31LL * nsm && n <= 8LL * 63 * nsm;
   int tile = mid ? 63 : default_tile(prob->flux, n);
 
   const Ctl h = make_ctl(cfl, dt_fixed, t_final);
@@ -919,8 +921,6 @@ int weno_theta_step(const wt_problem* prob, const wt_grid* grid, double* u, doub
   //   all tiles co-resident: the persistent kernel with a halo exchange per stage;
   //   otherwise: CUDA graphs of the three stage kernels of an RK step.
   const bool strict = prob->mode == WT_MODE_STRICT;
-  int nsm = 0;
-  WT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int tsb = stepblock1d_tile(prob->flux, n, nsm);
   const long long nsb = (n + tsb - 1) / tsb;
   long long ntiles = (n + tile - 1) / tile;

@@ -27,7 +27,7 @@ struct FluxM {
 // done, also holds the interface fluxes h of phase D and the window of u^n, which is copied in
 // after phase C1 (stages 2, 3) instead of with the stage input, so a tile needs about a sixth
 // less shared memory and one more tile fits on an SM.
-// DP (the fast policy's 1D Euler tiles, MATH::kDiffProj): the differences of f and u between
+// DP (the adjoint's forward tiles in fast mode, MATH::kDiffProj): the differences of f and u between
 // neighbouring cells, taken once per stage after phase C0; those of f go to the planes of the
 // per-cell Roe inputs (dead once phase C0 is done), those of u to planes of their own.
 template <int T, int M, int SPLIT = 1, int IPT = 1, bool LATE = false, bool DP = false>
@@ -50,12 +50,10 @@ struct Tile1D {
   static constexpr int kHf = LATE ? kL : kFs + 2 * M * NI;
   static constexpr int kUn = LATE ? kL + M * NI : kUin + M * W;
   static_assert(!LATE || (M * NI + M * W <= 9 * NI && (kUn % 2) == 0), "h and u^n fit the eigenvector buffer");
-  // (resident and step-blocked tiles, latency-bound: f's differences get planes of their own
-  // and are taken during phase C0)
   static constexpr int kDu = LATE ? kFs + 2 * M * NI : kHf + M * NI;  // DP: [M][W] u_{k+1} - u_k
-  static constexpr int kDf = LATE ? kVel : kDu + M * W;               // DP: [M][W] f_{k+1} - f_k
-  static_assert(!DP || M == 3, "differences first: 1D Euler tiles");
-  static constexpr int kRed = kDu + (DP ? (LATE ? 1 : 2) * M * W : 0);
+  static constexpr int kDf = kVel;                                    // DP: [M][W] f_{k+1} - f_k
+  static_assert(!DP || (M == 3 && LATE), "differences first: 1D Euler stage tiles");
+  static constexpr int kRed = kDu + (DP ? M * W : 0);
   static constexpr int kQn = kRed + 4 * 32;      // queue length (int)
   // queue of reconstructions still to be completed (DP; the screened scalar tiles list their
   // interfaces here): one slot per thread, fewer if the tile would pass 48 KB (the rest are
@@ -1040,7 +1038,7 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
   constexpr bool SCALAR = MATH::kCentral && FLUX != WT_FLUX_EULER1D;  // screened scalar tiles
   using TL = KernelTile<MATH, FLUX, T, MODE, IPT, USE>;
   constexpr int W = TL::W, NI = TL::NI, NT = TL::NT;
-  // differences first (phase C1): the adjoint's forward tiles (the central tiles' FP64 path does so too)
+  // differences first (phase C1): the adjoint's recording tiles (the central tiles' FP64 path does so too)
   constexpr bool DP = MATH::kDiffProj && FLUX == WT_FLUX_EULER1D && !CENTRAL;
   static_assert(!DP || (MODE == kStage && IPT > 1), "the adjoint's forward tiles");
   static_assert(NT * IPT >= SPLIT * M * NI, "IPT (interface, field) items per thread (one per thread pair with SPLIT = 2)");
@@ -1216,21 +1214,18 @@ __device__ __forceinline__ bool stage1d_compute(const Stage1DArgs& a, const long
     c0_barrier();
   }
   // DP: the differences of f and u between neighbouring window cells (f's over the per-cell
-  // Roe inputs, read for the last time in phase C0), by the threads of phase C0
+  // Roe inputs, read for the last time in phase C0)
   double* s_df = sm + TL::kDf;
   double* s_du = sm + TL::kDu;
   if constexpr (DP) {
-    if (!(sw_free && (tid >> 5) == kSW)) {
-      const int np = sw_free ? NT - 32 : NT;
-      for (int k = tid; k < cells - 1; k += np) {
+    for (int k = tid; k < cells - 1; k += NT) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          s_df[c * W + k] = s_f[c * W + k + 1] - s_f[c * W + k];
-          s_du[c * W + k] = s_uin[c * W + off + k + 1] - s_uin[c * W + off + k];
-        }
+      for (int c = 0; c < 3; ++c) {
+        s_df[c * W + k] = s_f[c * W + k + 1] - s_f[c * W + k];
+        s_du[c * W + k] = s_uin[c * W + off + k + 1] - s_uin[c * W + off + k];
       }
     }
-    c0_barrier();
+    __syncthreads();
   }
 
   // ---- C1: per (interface, field) reconstruction on both sides.  The projections onto the

@@ -366,12 +366,7 @@ struct FastMath {
   // value is the same as theirs.
   __device__ __forceinline__ static int weno_front_d(const double* d, double q2, double eps, double alpha_R,
                                                      double* rec) {
-    return weno_front_core<true>(d[0], d[1], d[2], d[3], d[4], q2, 0.0, eps, alpha_R, rec);
-  }
-  template <bool Q3D>
-  __device__ __forceinline__ static int weno_front_core(double d0, double d1, double d2, double d3, double d4,
-                                                        double q2, double q3, double eps, double alpha_R,
-                                                        double* rec) {
+    const double d0 = d[0], d1 = d[1], d2 = d[2], d3 = d[3], d4 = d[4];
     const double s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
     const double t5b = s2 - s1;
     const double t5a = fma(-2.0, s1, s0) + s2;
@@ -382,7 +377,7 @@ struct FastMath {
     rec[0] = d0; rec[1] = d1; rec[2] = d2; rec[3] = d3; rec[4] = d4;
     rec[5] = s0; rec[6] = s1; rec[7] = s2; rec[8] = s3;
     rec[9] = t5a; rec[10] = t5b; rec[11] = t6a; rec[12] = t6b;
-    rec[13] = q2; rec[14] = Q3D ? q2 + d2 : q3;
+    rec[13] = q2; rec[14] = q2 + d2;
     return 0;
   }
 
