@@ -84,6 +84,7 @@ struct TileC {
   // the central screen, 16.4)
   static constexpr bool kRoeWarp = kThree && T == 31 && MODE != kStepBlocked;
   static constexpr bool kRoeMemory = kRoeWarp && MODE == kResident;  // ... if the tile needed them in the last stage
+  static constexpr bool kSingles = MODE != kStage || T == 31;  // (central_deferred)
   static constexpr int NP = NT_;  // threads of the screen and of the FP64 path
   static constexpr int NT = NT_ + (kRoeWarp ? 32 : 0);
   static constexpr int FC = kThree ? (NI < 64 ? NI : 64) : (NI < 32 ? NI : 32);
@@ -383,9 +384,20 @@ __device__ __forceinline__ double central_flux(const double* sm, int c, int i) {
 // barrier 4 once the inputs are read.
 template <class MATH, class TL, bool AHEAD = false>
 __device__ __forceinline__ void central_roe(const Stage1DArgs& a, double* sm, int off, int i, int q) {
-  const double *pr = sm + TL::kUin + off + i + 2, *pv = sm + TL::kVel + i + 2, *pH = sm + TL::kH + i + 2;
-  const double r[2] = {pr[0], pr[1]}, v[2] = {pv[0], pv[1]}, H[2] = {pH[0], pH[1]};
-  if constexpr (AHEAD) named_barrier_arrive(4, TL::NT);
+  const double *r = sm + TL::kUin + off + i + 2, *v = sm + TL::kVel + i + 2, *H = sm + TL::kH + i + 2;
+  double c[6];
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      c[e] = r[e];
+      c[2 + e] = v[e];
+      c[4 + e] = H[e];
+    }
+    r = c;
+    v = c + 2;
+    H = c + 4;
+    named_barrier_arrive(4, TL::NT);
+  }
   double L[9], rs[3];
   double sa, sb;
   if constexpr (TL::kD != TL::kSr) {  // taken per cell in phase B
@@ -485,7 +497,8 @@ struct SidePair {
 };
 // the deferred stencils: a quad of lanes each (FastMath::weno_back_quad) where one round of the block holds
 // them, else a thread each (half the FP64 lane instructions; the same value): 28,001 cells of blast waves
-// 25.9 -> 23.4 us per stage with the longer queue
+// 25.9 -> 23.4 us per stage with the longer queue.  Not in the 63-cell stage tiles: the registers
+// (80 -> 96) would cost them one of four CTAs per SM (38,039 smooth cells 10.6 -> 11.9 ms for 200 steps).
 template <class MATH, class TL>
 __device__ __forceinline__ void central_deferred(const Stage1DArgs& a, double* sm) {
   const int nq = min(*reinterpret_cast<const int*>(sm + TL::kQn), TL::QCAP);
@@ -493,22 +506,26 @@ __device__ __forceinline__ void central_deferred(const Stage1DArgs& a, double* s
   auto put = [&](const int qi, const double v) {
     sm[TL::kFs + (qi & ((1 << 30) - 1))] = flip_sign(v, (qi >> 30) & 1 ? 0x8000000000000000ull : 0ull);
   };
-  if (4 * nq > TL::NP) {  // the same for every thread
-    for (int t = threadIdx.x; t < nq; t += TL::NP) {
-      double d[5];
+  if constexpr (TL::kSingles) {
+    if (4 * nq > TL::NP) {  // the same for every thread
+      for (int t = threadIdx.x; t < nq; t += TL::NP) {
+        double d[5];
 #pragma unroll
-      for (int y = 0; y < 5; ++y) d[y] = sm[TL::kQ + y * TL::QCAP + t];
-      put(s_qi[t], MATH::weno_d(d, sm[TL::kQ + 13 * TL::QCAP + t], a.eps, a.alpha_R));
+        for (int y = 0; y < 5; ++y) d[y] = sm[TL::kQ + y * TL::QCAP + t];
+        put(s_qi[t], MATH::weno_d(d, sm[TL::kQ + 13 * TL::QCAP + t], a.eps, a.alpha_R));
+      }
+      return;
     }
-    return;
   }
-  const int t = (int)threadIdx.x >> 2, z = threadIdx.x & 3;
-  if (t < nq) {  // the same for the four lanes of a quad
-    double rec[TL::REC];
+  for (int b0 = 0; b0 < nq; b0 += TL::NP / 4) {
+    const int t = b0 + ((int)threadIdx.x >> 2), z = threadIdx.x & 3;
+    if (t < nq) {  // the same for the four lanes of a quad
+      double rec[TL::REC];
 #pragma unroll
-    for (int y = 0; y < TL::REC; ++y) rec[y] = sm[TL::kQ + y * TL::QCAP + t];
-    const double out = MATH::weno_back_quad(z, rec, a.eps, a.alpha_R, 0xfu << (threadIdx.x & 28));
-    if (z == 0) put(s_qi[t], out);
+      for (int y = 0; y < TL::REC; ++y) rec[y] = sm[TL::kQ + y * TL::QCAP + t];
+      const double out = MATH::weno_back_quad(z, rec, a.eps, a.alpha_R, 0xfu << (threadIdx.x & 28));
+      if (z == 0) put(s_qi[t], out);
+    }
   }
 }
 
