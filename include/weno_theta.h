@@ -201,7 +201,8 @@ int weno_theta_step_batched(const wt_problem* prob, const wt_segment* segs, int3
  *   uT      [nprob][3][n] out (may be NULL): u(T), bit for bit as the step entry points return it.  In
  *           WT_MODE_FAST those evaluate smooth interfaces without the characteristic projections
  *           (to rounding the same flux), which the differentiated pass keeps: asking for uT
- *           then runs the steps once more
+ *           then runs the steps once more, 7 to 8 % of the call (256 problems of 16384 cells,
+ *           64 steps); uT = NULL where the caller has u(T) already
  * prob->flux must be WT_FLUX_EULER1D.  ws must hold wt_adjoint_workspace_bytes(...) bytes.
  * The environment variable WT_ADJ_TILE (31, 2031, 63, 1063 or 2063: cells per reverse tile +
  * 1000 x (items per thread - 1)) overrides the reverse kernel's tile; the gradients agree to

@@ -2,8 +2,11 @@
 
 ``WenoThetaEuler1D.apply(u0, ...)`` advances nprob independent 1D Euler problems
 (``u0``: CUDA float64 tensor ``[nprob, 3, n]``) by ``n_steps`` TVD-RK3 steps with the
-WENO-theta scheme; its backward pass calls ``weno_theta_adjoint`` (reverse mode of the exact
-map, branches frozen as the forward took them, checkpoints every ``checkpoint_every`` steps).
+WENO-theta scheme; its backward pass calls ``weno_theta_adjoint`` (reverse mode of the steps, run
+again with every flux projected and each branch frozen as that pass takes it; checkpoints every
+``checkpoint_every`` steps).  In ``WT_MODE_FAST`` the projected pass agrees with the returned
+state to rounding, so a branch that is decided at the level of rounding alone (theta where a
+field is constant) need not be the one the returned state took.
 Both directions run in the CUDA library; this module only allocates workspaces and marshals.
 """
 from __future__ import annotations

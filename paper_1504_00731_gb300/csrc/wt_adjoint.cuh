@@ -1,7 +1,8 @@
-// Discrete adjoint of the 1D Euler hot path (reverse mode of the exact map the forward pass
-// computes).  Every branch is frozen where the forward pass took it: theta and the
-// restriction of each reconstruction are re-decided by the same arithmetic policy as the
-// forward, and the derivative of each maximum (the Lax-Friedrichs alphas, the CFL step)
+// Discrete adjoint of the 1D Euler hot path (reverse mode of the exact map its own forward pass
+// computes: the stages with every reconstruction projected).  Every branch is frozen where that
+// pass took it: theta and the restriction of each reconstruction are read from its records
+// (fast mode: the step entry points agree with it to rounding, so that branches taken on rounding
+// noise may differ from theirs), and the derivative of each maximum (the Lax-Friedrichs alphas, the CFL step)
 // goes to the first cell that attains it.
 //
 //   adj_stage_kernel   one RK stage in reverse over a tile: recomputes the stage's interface

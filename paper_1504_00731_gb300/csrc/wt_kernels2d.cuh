@@ -49,9 +49,8 @@ struct Tile2D {
   static_assert(2 * (bytes + 1024) <= 228 * 1024, "two tiles must fit on one SM");
 };
 
-// What the fast policy's kernel costs: about 190 FP64 thread instructions per cell and stage where the data
-// are smooth (1245 with every interface projected), 58 % of the FP64 pipe's cycles at 16 warps per
-// SM; 2048 x 2048 vortices 59.8 -> 17.4 ms for two steps, 120 x 360 Rayleigh-Taylor 22.3 -> 11.5
+// What the fast policy's kernel costs: 230 FP64 thread instructions per cell and stage on 1024 x 1024
+// vortices (1245 with every interface projected), 53 % of the FP64 pipe's cycles at 16 warps per SM; 2048 x 2048 vortices 59.8 -> 17.4 ms for two steps, 120 x 360 Rayleigh-Taylor 22.3 -> 11.5
 // ms for 40 (a fifth of its y interfaces are on fronts and take the FP64 path).
 //
 // Tile of the central screen (wt_central.cuh; the fast policy): no eigenvector or reconstruction
